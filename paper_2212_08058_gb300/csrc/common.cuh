@@ -59,34 +59,59 @@ __device__ __forceinline__ double warp_sum(double v) {
     return v;
 }
 
-// Sum of `v` over the block (any blockDim that is a multiple of 32, at most 1024).
-// All threads must call it; the result is valid in thread 0.
+// Sum of `v` over the block (blockDim a multiple of 32, at most 256).  All threads must call it;
+// the result is valid in thread 0.
+// FP64 runs at 2 FMA per clock per SM here, 1/64 of FP32: a butterfly in every warp costs 5 FP64
+// additions per warp, 45 for 256 threads, 16 clocks each (about 2.5 us for an SM's eight blocks).
+// So the partial sums go through shared memory and one warp adds them: 12 for 256 threads.
 __device__ __forceinline__ double block_sum(double v) {
-    __shared__ double red[32];
-    v = warp_sum(v);
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    __shared__ double red[256];
     __syncthreads();   // protects red[] against a previous call
-    if (lane == 0) red[wid] = v;
+    red[threadIdx.x] = v;
     __syncthreads();
     double r = 0.0;
-    if (wid == 0) {
-        const int nw = (blockDim.x + 31) >> 5;
-        r = lane < nw ? red[lane] : 0.0;
+    if (threadIdx.x < 32) {
+        r = red[threadIdx.x];
+        for (int i = threadIdx.x + 32; i < (int)blockDim.x; i += 32) r += red[i];
         r = warp_sum(r);
     }
     return r;
 }
 
 // 1/sqrt(acc) of an FP64 sum of squares, with the flag raised (and 0 returned) when the sum is
-// zero or not finite, so that later iterations produce zeros instead of NaNs.
+// zero or not finite, so that later iterations produce zeros instead of NaNs.  For one thread of
+// a block (block_inv_norm gives it to all): an FP64 square root and division in every thread of a
+// launch cost more than many of the launches' own work (3.3M voxels, 2432 x 256 threads: 25 us of
+// a 28.6 us pass).  Within float's range the reciprocal square root is one FP64 Newton step from
+// the FP32 one (relative error below 2^-43 before the rounding to float).
 __device__ __forceinline__ float inv_norm_from(const double* acc, int* flags) {
     if (acc == nullptr) return 1.f;
     const double a = *acc;
+    if (a > 1e-30 && a < 1e30) {
+        const double y = (double)rsqrtf((float)a);
+        const double e = fma(-a * y, y, 1.0);
+        return (float)fma(0.5 * y, e, y);
+    }
     if (!(a > 0.0) || !(a < 1e300)) {
-        if (threadIdx.x == 0 && flags) atomicOr(flags, a == 0.0 ? kFlagZeroNorm : kFlagNonfinite);
+        if (flags) atomicOr(flags, a == 0.0 ? kFlagZeroNorm : kFlagNonfinite);
         return 0.f;
     }
     return (float)(1.0 / sqrt(a));
+}
+
+// f() of one thread given to the whole block; every thread must call it.  `I` tells the calls of
+// one kernel apart (each has its own shared word).
+template <int I = 0, typename F>
+__device__ __forceinline__ float block_value(F&& f) {
+    __shared__ float value;
+    if (threadIdx.x == 0) value = f();
+    __syncthreads();
+    return value;
+}
+
+template <int I = 0>
+__device__ __forceinline__ float block_inv_norm(const double* acc, int* flags) {
+    return block_value<I>([&] { return inv_norm_from(acc, flags); });
 }
 
 }  // namespace sfseg

@@ -39,9 +39,9 @@ struct OpAdjoint {
     float sk, sn, dotn;
 
     __device__ __forceinline__ void begin(const double*, int* flags) {
-        sk = inv_norm_from(acc_k, flags);
-        sn = inv_norm_from(acc_n, flags);
-        dotn = (float)*dot_n;
+        sk = block_inv_norm<0>(acc_k, flags);
+        sn = block_inv_norm<1>(acc_n, flags);
+        dotn = block_value<2>([&] { return (float)*dot_n; });
     }
     __device__ __forceinline__ void xg(int64_t i, float& x, float& gy) const {
         x = sk * xk[i];
@@ -114,8 +114,8 @@ __global__ void state_internal_kernel(const float* x, const float* f, float p, G
 // v_g of the first reverse step: u g_y = s_K u (g_K - s_K x~_K <x_K, g_K>).
 __global__ void adjoint_first_kernel(const float* xK, const double* accK, const float* gK, const double* dotK,
                                      const float* f, float p, Geom g, float* vg) {
-    const float sK = inv_norm_from(accK, nullptr);
-    const float d = (float)*dotK;
+    const float sK = block_inv_norm<0>(accK, nullptr);
+    const float d = block_value<1>([&] { return (float)*dotK; });
     for_each_voxel(g, [&](int64_t, int64_t j) {
         vg[j] = unary_pow_fast(f[j], p) * ((gK[j] - sK * xK[j] * d) * sK);
     });
@@ -134,8 +134,8 @@ void launch_adjoint_first(const float* xK, const double* accK, const float* gK, 
 __global__ void adjoint_combine_state_kernel(const float* f, const float* vg, const float* qx, const float* Vk,
                                              const float* qg, const float* Gk, const double* acc_k,
                                              const double* dsum, Geom g, float* gz, float* vg_next) {
-    const float sk = inv_norm_from(acc_k, nullptr);
-    const float dot = sk * (float)*dsum;
+    const float sk = block_inv_norm<0>(acc_k, nullptr);
+    const float dot = sk * block_value<1>([&] { return (float)*dsum; });
     // rows (t, h) over the blocks, four columns per thread (internal rows start 128-byte
     // aligned), the ragged end of a row one column at a time
     const int64_t rows = (int64_t)g.T * g.H;
@@ -193,58 +193,57 @@ void launch_state_internal(const float* x, const float* f32, float p, Geom g, fl
 // g_K from the caller's layout into the internal layout, and <x_K, g_K>.
 __global__ void grad_in_kernel(const float* gx_user, const float* xK, const double* accK, float* g_out, Geom g,
                                double* dot_out) {
-    const float sK = inv_norm_from(accK, nullptr);
-    const int64_t HW = (int64_t)g.H * g.W, N = HW * g.T;
+    const float sK = block_inv_norm(accK, nullptr);
     float part = 0.f;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t t = i / HW, rem = i - t * HW;
-        const int64_t h = rem / g.W, wc = rem - h * g.W;
-        const int64_t j = (t * g.H + h) * g.pitch + wc;
+    for_each_voxel(g, [&](int64_t i, int64_t j) {
         const float gv = gx_user[i];
         g_out[j] = gv;
         part += sK * xK[j] * gv;
-    }
+    });
     const double b = block_sum((double)part);
     if (threadIdx.x == 0) atomicAdd(dot_out, b);
 }
 
 void launch_grad_in(const float* gx_user, const float* xK, const double* accK, float* g_out, Geom g,
                     double* dot_out, cudaStream_t s) {
-    const int64_t N = (int64_t)g.T * g.H * g.W;
-    int blocks = (int)((N + 255) / 256);
-    if (blocks > 8 * num_sms()) blocks = 8 * num_sms();
-    grad_in_kernel<<<blocks, 256, 0, s>>>(gx_user, xK, accK, g_out, g, dot_out); count_launches(1);
+    const RowLaunch rl = row_launch(g, num_sms(), 8);
+    grad_in_kernel<<<rl.blocks, rl.threads, 0, s>>>(gx_user, xK, accK, g_out, g, dot_out);
+    count_launches(1);
 }
 
-// acc[c] += sum_i gz_i V_c,i  (c < C),  acc[C] += sum_i gz_i.
+// acc[c] += sum_i gz_i V_c,i  (c < C),  acc[C] += sum_i gz_i.  Eight channels per pass over gz, so
+// that the partial sums stay in registers; the passes after the first re-read gz (from L2).
 template <typename TIn>
 __global__ void weight_grad_kernel(const TIn* feat, int C, Geom g, const float* gz, double* acc) {
-    constexpr int kMaxC = 64;
-    float part[kMaxC + 1];
-    for (int c = 0; c <= C; ++c) part[c] = 0.f;
-    const int64_t HW = (int64_t)g.H * g.W, N = HW * g.T;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t t = i / HW, rem = i - t * HW;
-        const int64_t h = rem / g.W, wc = rem - h * g.W;
-        const float gv = gz[(t * g.H + h) * g.pitch + wc];
-        part[C] += gv;
-        for (int c = 0; c < C; ++c) part[c] += gv * ldf(feat + (int64_t)c * N + i);
-    }
-    for (int c = 0; c <= C; ++c) {
-        const double b = block_sum((double)part[c]);
-        if (threadIdx.x == 0) atomicAdd(acc + c, b);
+    constexpr int kC = 8;
+    const int64_t N = (int64_t)g.T * g.H * g.W;
+    for (int c0 = 0; c0 < C; c0 += kC) {
+        float part[kC + 1];
+#pragma unroll
+        for (int c = 0; c <= kC; ++c) part[c] = 0.f;
+        for_each_voxel(g, [&](int64_t i, int64_t j) {
+            const float gv = gz[j];
+            part[kC] += gv;
+#pragma unroll
+            for (int c = 0; c < kC; ++c)
+                if (c0 + c < C) part[c] += gv * ldf(feat + (int64_t)(c0 + c) * N + i);
+        });
+#pragma unroll
+        for (int c = 0; c <= kC; ++c) {
+            if (c < kC ? c0 + c >= C : c0 > 0) continue;
+            const double b = block_sum((double)part[c]);
+            if (threadIdx.x == 0) atomicAdd(acc + (c < kC ? c0 + c : C), b);
+        }
     }
 }
 
 void launch_weight_grad(const void* feat, int feat_dtype, int C, Geom g, const float* gz, double* acc,
                         cudaStream_t s) {
-    const int64_t N = (int64_t)g.T * g.H * g.W;
-    int blocks = (int)((N + 255) / 256);
-    if (blocks > 4 * num_sms()) blocks = 4 * num_sms();
+    const RowLaunch rl = row_launch(g, num_sms(), 4);
     if (feat_dtype == kF32)
-        weight_grad_kernel<float><<<blocks, 256, 0, s>>>((const float*)feat, C, g, gz, acc);
+        weight_grad_kernel<float><<<rl.blocks, rl.threads, 0, s>>>((const float*)feat, C, g, gz, acc);
     else
-        weight_grad_kernel<__nv_bfloat16><<<blocks, 256, 0, s>>>((const __nv_bfloat16*)feat, C, g, gz, acc);
+        weight_grad_kernel<__nv_bfloat16><<<rl.blocks, rl.threads, 0, s>>>((const __nv_bfloat16*)feat, C, g, gz, acc);
     count_launches(1);
 }
 
@@ -293,8 +292,8 @@ __global__ void iou_sums_kernel(const float* x, const float* tg, int64_t n, cons
 __global__ void iou_grad_kernel(const float* x, const float* tg, int64_t n, const unsigned long long* amax,
                                 double* acc, float* grad) {
     const float m = key_value(*amax);
-    const double I = acc[0], U = acc[1];
-    const float cu = (float)(1.0 / U), ci = (float)(I / (U * U));
+    const float cu = block_value<0>([&] { return (float)(1.0 / acc[1]); });
+    const float ci = block_value<1>([&] { return (float)(acc[0] / (acc[1] * acc[1])); });
     float a = 0.f;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const float gv = tg[i];

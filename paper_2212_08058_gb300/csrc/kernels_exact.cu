@@ -24,7 +24,7 @@ __global__ void exact_in_kernel(const float* x_user, Geom g, float* xt, double* 
 // v = f^{3j} s u e^{-a f^2} x~, s = 1/sqrt(*acc) (1 if acc is null).
 __global__ void exact_prep_kernel(const float* xt, const double* acc, const float* f, float alpha, float p, int jt,
                                   Geom g, float* v, int* flags) {
-    const float s = inv_norm_from(acc, flags);
+    const float s = block_inv_norm(acc, flags);
     for_each_voxel(g, [&](int64_t, int64_t j) {
         const float fv = f[j];
         const float f3 = fv * fv * fv;
@@ -36,7 +36,7 @@ __global__ void exact_prep_kernel(const float* xt, const double* acc, const floa
 
 // The caller's x = s y (y internal), s = 1/sqrt(*acc) (1 if acc is null).
 __global__ void exact_out_kernel(const float* y, const double* acc, Geom g, float* x_user, int* flags) {
-    const float s = inv_norm_from(acc, flags);
+    const float s = block_inv_norm(acc, flags);
     for_each_voxel(g, [&](int64_t i, int64_t j) { x_user[i] = s * y[j]; });
 }
 

@@ -97,6 +97,34 @@ __device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, u
         : "memory");
 }
 
+// common.cuh's block_sum and inv_norm_from in the forms that leave this kernel's register
+// allocation as it is: at (2,7,7) the shared ones cost 0.9 % of the step (its 168 registers are all
+// taken), and the FP64 work they save is hidden behind the first copies.
+__device__ __forceinline__ double tile_block_sum(double v) {
+    __shared__ double red[32];
+    v = warp_sum(v);
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    __syncthreads();   // protects red[] against a previous call
+    if (lane == 0) red[wid] = v;
+    __syncthreads();
+    double r = 0.0;
+    if (wid == 0) {
+        const int nw = (blockDim.x + 31) >> 5;
+        r = lane < nw ? red[lane] : 0.0;
+        r = warp_sum(r);
+    }
+    return r;
+}
+__device__ __forceinline__ float tile_inv_norm(const double* acc, int* flags) {
+    if (acc == nullptr) return 1.f;
+    const double a = *acc;
+    if (!(a > 0.0) || !(a < 1e300)) {
+        if (threadIdx.x == 0 && flags) atomicOr(flags, a == 0.0 ? kFlagZeroNorm : kFlagNonfinite);
+        return 0.f;
+    }
+    return (float)(1.0 / sqrt(a));
+}
+
 __device__ __forceinline__ float2 f2(float a) { return make_float2(a, a); }
 __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
 __device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
@@ -200,7 +228,7 @@ iter_fast(const __grid_constant__ CUtensorMap mv, const __grid_constant__ CUtens
     // streamed, to flush the last rt output frames.
     const int tstart = max(t0 - RT, 0), tend = t1 + RT;
 
-    const float s = inv_norm_from(P.acc_in, P.flags);
+    const float s = tile_inv_norm(P.acc_in, P.flags);
     const float2 s2 = f2(s);
 
     if (tid == 0) {
@@ -507,7 +535,7 @@ iter_fast(const __grid_constant__ CUtensorMap mv, const __grid_constant__ CUtens
         }
         return;
     }
-    const double tot = block_sum((double)part.x + (double)part.y);
+    const double tot = tile_block_sum((double)part.x + (double)part.y);
     if (tid == 0 && P.acc_out) atomicAdd(P.acc_out, tot);
     if constexpr (MODE == 8) {
         __shared__ unsigned wmax[NTHR / 32];

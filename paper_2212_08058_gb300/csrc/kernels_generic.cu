@@ -41,7 +41,7 @@ struct OpIter {
     float inv_alpha, p, s;
 
     __device__ __forceinline__ void begin(const double* acc_in, int* flags) {
-        s = inv_norm_from(acc_in, flags);
+        s = block_inv_norm(acc_in, flags);
     }
     __device__ __forceinline__ void load(int t, int h, int w, float (&z)[NS]) const {
         const int64_t i = ((int64_t)t * g.H + h) * g.pitch + w;
@@ -78,7 +78,7 @@ struct OpApply {
     float inv_alpha, p, s;
 
     __device__ __forceinline__ void begin(const double* acc_in, int* flags) {
-        s = inv_norm_from(acc_in, flags);
+        s = block_inv_norm(acc_in, flags);
     }
     __device__ __forceinline__ void load(int t, int h, int w, float (&z)[NS]) const {
         const float xv = x[((int64_t)t * g.H + h) * x_pitch + w];
@@ -360,7 +360,7 @@ void launch_to_bf16(const float* a, __nv_bfloat16* b, int64_t n, cudaStream_t s)
 
 // ------------------------------------------------------------------------- reductions
 __global__ void scale_inv_norm_kernel(float* x, int64_t n, bool vec, const double* acc, int* flags) {
-    const float s = inv_norm_from(acc, flags);
+    const float s = block_inv_norm(acc, flags);
     for_each_flat(
         n, vec,
         [&](int64_t i) {
@@ -397,7 +397,7 @@ __global__ void dot2_kernel(const float* x, const float* y, int64_t n, bool vec,
 }
 
 __global__ void resid_kernel(const float* x, const float* y, int64_t n, bool vec, double* acc) {
-    const float rho = (float)(acc[0] / acc[1]);
+    const float rho = block_value([&] { return (float)(acc[0] / acc[1]); });
     float a = 0.f;
     for_each_flat(
         n, vec,

@@ -873,10 +873,19 @@ __global__ void wgrad_reduce(const float* part, int nparts, int cout, int cin, f
             n = NCO * 8 + co;
             m = 96;
         }
-        double acc = 0.0;
-        for (int p = 0; p < nparts; ++p) acc += (double)part[(size_t)p * C::PART + ((size_t)dw * C::N + n) * 128 + m];
-        if (idx < total) dW[idx] = (float)acc;
-        else db[idx - total] = (float)acc;
+        // hi + lo: the error-free transformation of each addition (Knuth's TwoSum), which keeps the
+        // sum to about 48 bits like FP64 would, at FP32 rate
+        float hi = 0.f, lo = 0.f;
+#pragma unroll 8
+        for (int p = 0; p < nparts; ++p) {
+            const float v = part[(size_t)p * C::PART + ((size_t)dw * C::N + n) * 128 + m];
+            const float t = __fadd_rn(hi, v), z = __fsub_rn(t, hi);
+            lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(t, z)), __fsub_rn(v, z)));
+            hi = t;
+        }
+        const float acc = hi + lo;
+        if (idx < total) dW[idx] = acc;
+        else db[idx - total] = acc;
     }
 }
 
@@ -948,9 +957,9 @@ __global__ void cos_sums(const float* x, const float* g, int64_t n, double* acc)
 // tensor (the input of the last layer's data-gradient convolution), other channels zero.
 __global__ void cos_grad(const float* x, const float* g, const float* z, int64_t n, const double* acc,
                          __nv_bfloat16* dz16) {
-    const double xg = acc[0], xx = acc[1], gg = acc[2];
-    const double nx = sqrt(xx), ng = sqrt(gg);
-    const float c1 = (float)(1.0 / (nx * ng)), c2 = (float)(xg / (nx * ng) / xx);
+    // acc: sums of x*g, x*x, g*g
+    const float c1 = block_value<0>([&] { return (float)(1.0 / (sqrt(acc[1]) * sqrt(acc[2]))); });
+    const float c2 = block_value<1>([&] { return (float)(acc[0] / (sqrt(acc[1]) * sqrt(acc[2])) / acc[1]); });
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const float dx = -(g[i] * c1 - x[i] * c2);
         const float sg = 1.f / (1.f + expf(-z[i]));
