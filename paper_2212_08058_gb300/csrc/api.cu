@@ -781,7 +781,7 @@ int sfseg_backward(sfseg_handle* h, const sfseg_neighborhood* nb, const float* g
     for (int i = 0; i < 2; ++i)
         if (!h->gbuf[i]) SFSEG_CUDA(dalloc(&h->gbuf[i], (size_t)h->NP));
     if (!h->gz) SFSEG_CUDA(dalloc(&h->gz, (size_t)h->NP));
-    const bool fast_adj = fast_iterate_supported(tp);
+    const bool fast_adj = fast_step_supported(tp);
     if (fast_adj)
         for (float*& q : h->adjw)
             if (!q) SFSEG_CUDA(dalloc(&q, (size_t)h->NP));
@@ -824,7 +824,7 @@ int sfseg_backward(sfseg_handle* h, const sfseg_neighborhood* nb, const float* g
                         return fail(SFSEG_ERR_CUDA, "the TMA stencil could not be launched");
                     SFSEG_LAUNCHED();
                 }
-                if (!launch_filter_fast(h->seg[n - 1], 1, h->qxs[n - 1], nullptr, h->f32, h->g, tp, inv_alpha, p,
+                if (!launch_filter_fast(h->seg[n - 1], h->qxs[n - 1], h->f32, h->g, tp, inv_alpha, p,
                                         h->rec_acc + k1 - 1, h->flags, st))
                     return fail(SFSEG_ERR_CUDA, "the TMA stencil could not be launched");
                 SFSEG_LAUNCHED();
@@ -1020,7 +1020,7 @@ int sfseg_soft_binarize(sfseg_handle* h, const sfseg_neighborhood* nb, int iters
     float* y = (float*)h->vbuf[0];                     // A x, caller layout
     float* v = (float*)h->vbuf[1];                     // u * x, internal layout
     unsigned* key = reinterpret_cast<unsigned*>(h->scratch + kScrMaxKey);
-    const bool fast = fast_iterate_supported(tp);
+    const bool fast = fast_step_supported(tp);
     const float* s32 = h->sep ? h->s32 : nullptr;
     for (int k = 0; k < iters; ++k) {
         const bool last = k == iters - 1;

@@ -45,11 +45,12 @@ __device__ __forceinline__ float unary_pow(float s, float p) {
 
 // Faster variant on the special-function unit: u = 2^(p log2 s) with the approximate log2 and
 // exp2 instructions (relative error a few 1e-7 for p <= 1).  s = 0 gives log2 s = -inf and
-// u = +0, so no branch is needed (s < 0 never reaches here: features are checked >= 0).
+// u = +0, so no branch is needed (s < 0 never reaches here: features are checked >= 0).  lg2 takes
+// subnormal s (its u is not small); u itself below 2^-126 becomes 0 (three instructions less).
 __device__ __forceinline__ float unary_pow_fast(float s, float p) {
     float l, u;
     asm("lg2.approx.f32 %0, %1;" : "=f"(l) : "f"(s));
-    asm("ex2.approx.f32 %0, %1;" : "=f"(u) : "f"(p * l));
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(u) : "f"(p * l));
     return u;
 }
 

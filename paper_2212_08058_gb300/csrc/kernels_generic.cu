@@ -108,11 +108,15 @@ static std::atomic<int64_t> g_steps_tma{0}, g_steps_generic{0};
 static std::mutex g_step_mu;
 static char g_step_name[96] = "";
 
+// `tma`: the step ran on the TMA kernels.  Steps of a radius without its own kernel count as generic
+// ones, whether they ran on a TMA kernel of a wider radius with zero taps or on stream_stencil.
 static void note_step(bool tma, const Taps& tp, int vin_type, int out_type, bool out_x, bool record, bool sep) {
-    (tma ? g_steps_tma : g_steps_generic).fetch_add(1, std::memory_order_relaxed);
+    const bool own = tma && fast_iterate_supported(tp);
+    (own ? g_steps_tma : g_steps_generic).fetch_add(1, std::memory_order_relaxed);
     char buf[96];
-    std::snprintf(buf, sizeof(buf), "%s<%d,%d,%d,%s,%s%s%s>", tma ? "iter_fast" : "stream_stencil<OpIter>", tp.rt,
-                  tp.rh, tp.rw, vin_type == kF32 ? "float" : "bf16",
+    std::snprintf(buf, sizeof(buf), "%s<%d,%d,%d,%s,%s%s%s>",
+                  own ? "iter_fast" : (tma ? "stream_stencil(padded taps)" : "stream_stencil<OpIter>"), tp.rt, tp.rh,
+                  tp.rw, vin_type == kF32 ? "float" : "bf16",
                   out_x ? "float(caller x)" : (out_type == kBF16 ? "bf16" : "float"), record ? ",record" : "",
                   sep ? ",separate maps" : "");
     std::lock_guard<std::mutex> lk(g_step_mu);
@@ -164,13 +168,13 @@ void launch_iterate(const void* vin, int vin_type, void* out, int out_type, bool
                     const double* acc_in, double* acc_out, int* flags, cudaStream_t s, const float* s32) {
     using bf = __nv_bfloat16;
     // The TMA kernel serves the method's radii, recording steps (float32, shared maps) included.
-    if (ckpt == nullptr && fast_iterate_supported(tp) &&
+    if (ckpt == nullptr && fast_step_supported(tp) &&
         launch_iterate_fast(vin, vin_type, out, out_type, out_x, f, g, tp, inv_alpha, p, acc_in, acc_out, flags, s,
                             s32)) {
         note_step(true, tp, vin_type, out_type, out_x, false, s32 != nullptr);
         return;
     }
-    if (ckpt != nullptr && vin_type == kF32 && s32 == nullptr && fast_iterate_supported(tp) &&
+    if (ckpt != nullptr && vin_type == kF32 && s32 == nullptr && fast_step_supported(tp) &&
         launch_iterate_fast_ckpt((const float*)vin, out, out_x, (const float*)f, g, tp, inv_alpha, p, acc_in, acc_out,
                                  ckpt, flags, s)) {
         note_step(true, tp, vin_type, out_type, out_x, true, false);
@@ -233,7 +237,7 @@ void launch_to_state(const float* x, const float* f32, const float* s32, float p
 
 void launch_apply_user(const float* x, float* y, float* scratch_v, const float* f32, Geom g, const Taps& tp,
                        float inv_alpha, float p, int* flags, cudaStream_t s, const float* s32) {
-    if (fast_iterate_supported(tp)) {
+    if (fast_step_supported(tp)) {
         const RowLaunch rl = row_launch(g, num_sms());
         to_state_kernel<<<rl.blocks, rl.threads, 0, s>>>(x, f32, s32, p, g, g.W % 2 == 0 && aligned8(x), scratch_v);
         count_launches(1);

@@ -40,6 +40,8 @@ void launch_iterate(const void* vin, int vin_type, void* out, int out_type, bool
 // (nullable): a separate unary map (float32 storage only).  Returns false when the radius has no
 // compiled kernel or a tensor map cannot be encoded; nothing is launched then.
 bool fast_iterate_supported(const Taps& tp);
+// The same, or a wider radius's kernel can run tp padded with zero taps.
+bool fast_step_supported(const Taps& tp);
 bool launch_iterate_fast(const void* vin, int vin_type, void* out, int out_type, bool out_x, const void* f,
                          const Geom& g, const Taps& tp, float inv_alpha, float p, const double* acc_in,
                          double* acc_out, int* flags, cudaStream_t s, const float* s32 = nullptr);
@@ -62,10 +64,10 @@ bool launch_iterate_fast_ckpt(const float* vin, void* out, bool out_x, const flo
 
 // The adjoint's Q-pass on the TMA kernel (kernels_fast.cu, mode 1), float32, internal layout:
 // for the signals c0, c1, c2 of v (G*v, G*(f^2 v), G*(f v)), writes Q = s (a1 c0 - p c1 + a3 c2)
-// to out, s = 1/sqrt(*acc_in) (or 1).  Returns false (nothing launched) for another mode or a
-// radius without a compiled kernel.
-bool launch_filter_fast(const float* vin, int mode, float* out, float* out2, const float* f, const Geom& g,
-                        const Taps& tp, float inv_alpha, float p, const double* acc_in, int* flags, cudaStream_t s);
+// to out, s = 1/sqrt(*acc_in) (or 1).  Returns false (nothing launched) for a radius that no
+// compiled kernel covers.
+bool launch_filter_fast(const float* vin, float* out, const float* f, const Geom& g, const Taps& tp, float inv_alpha,
+                        float p, const double* acc_in, int* flags, cudaStream_t s);
 
 // One term j of the exact (Eq. 1) kernel's series on the TMA kernel (kernels_fast.cu, mode 7):
 // for the input v = f^{3j} w (internal layout), adds the terms n = 3j, 3j+1, 3j+2 of

@@ -1,0 +1,10 @@
+// step_2_7_7.cu -- the Eq. 7 step's kernels for radius (2, 7, 7).
+#include "iter_stream.cuh"
+#include "iter_tile.cuh"
+
+namespace sfseg {
+
+bool stream_step_2_7_7(const StepArgs& a) { return step_dispatch<stream::Kernel<2, 7, 7>>(a); }
+bool tile_step_2_7_7(const StepArgs& a) { return step_dispatch<tile::Kernel<2, 7, 7>>(a); }
+
+}  // namespace sfseg

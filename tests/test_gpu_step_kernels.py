@@ -1,0 +1,86 @@
+"""The two kernels of the Eq. 7 step (csrc/iter_stream.cuh for volumes of at least 6 frames and 3.5
+output frames per SM, csrc/iter_tile.cuh below) and the radii that run on a wider radius's kernel with
+zero taps, at the sizes where they can go wrong: one row, column or frame past a tile, fewer tiles than
+SMs and more, tiles cut in time, both sides of the line between the kernels.
+
+Reference: the FP64 oracle.  Bound: an iterate of K steps is K times (2 rt + 1) + (2 rh + 1) + (2 rw + 1)
++ 12 roundings of positive float32 sums away from it, each 2^-24 of max x: 4 steps at (2,7,7) 4 * 47 *
+2^-24 = 1.1e-5 of max x."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def sf():
+    from paper_2212_08058_gb300 import build, sfseg
+    build.build()
+    oracle.build()
+    return sfseg
+
+
+def _check(sf, T, H, W, radius, seed, iters=4, bf16=0, init="uniform"):
+    rng = np.random.default_rng(seed)
+    V = rng.random((1, T, H, W)).astype(np.float32)
+    with sf.PowerIteration(1, T, H, W) as h:
+        x, nu = h.power_iterate(torch.from_numpy(V).cuda(), radius=radius, iters=iters, iters_bf16=bf16, init=init,
+                                return_norms=True)
+    f = V[0].astype(np.float64)
+    xo, nuo = oracle.power_filter(f, f, 0.1, 1.0, radius, f if init == "smap" else np.ones(f.shape), iters)
+    tol = 2e-2 if bf16 else iters * (2 * sum(radius) + 3 + 12) * 2.0 ** -24
+    assert np.abs(x.cpu().numpy() - xo).max() <= tol * xo.max(), (T, H, W, radius)
+    np.testing.assert_allclose(nu, nuo, rtol=tol)
+
+
+# tiles of 18 x 112 on 152 SMs: (6, 19 x 18, 5 x 112) is 95 tiles of 6 frames, 570 >= 532 output frames
+@pytest.mark.parametrize("T,H,W", [
+    (6, 342, 560), (6, 343, 561), (7, 341, 559),     # fewer tiles than SMs, cut in time
+    (6, 324, 1008), (6, 325, 1009),                  # 162 and 190 tiles: whole ones and a rest that is cut
+    (6, 144, 2128),                                  # 152 tiles: whole ones only
+    (6, 306, 1904), (540, 17, 113), (300, 1, 300),   # two whole tiles per block and a rest; long and flat
+    (6, 342, 336), (5, 342, 1008),                   # below the line: too few frames per SM, too short
+])
+@pytest.mark.parametrize("radius", [(1, 3, 3), (2, 7, 7)])
+def test_stream_and_tile_kernels(sf, T, H, W, radius):
+    _check(sf, T, H, W, radius, seed=T + H + W)
+
+
+@pytest.mark.parametrize("radius", [(0, 0, 0), (0, 1, 1), (1, 1, 1), (1, 6, 6), (2, 4, 4), (2, 2, 5), (0, 8, 0),
+                                    (1, 8, 8), (2, 8, 8), (2, 0, 8)])
+@pytest.mark.parametrize("T,H,W", [(7, 20, 113), (9, 343, 561)])
+def test_padded_radii(sf, radius, T, H, W):
+    _check(sf, T, H, W, radius, seed=17, init="smap")
+    assert sf.iterate_kernel_stats()[2].startswith("stream_stencil")
+
+
+def test_bf16_storage_in_the_stream_kernel(sf):
+    _check(sf, 6, 343, 561, (2, 7, 7), seed=3, iters=3, bf16=2)
+
+
+@pytest.mark.parametrize("T,H,W", [(7, 20, 113), (9, 343, 561)])
+def test_padded_radius_adjoint(sf, T, H, W):
+    """The adjoint of a padded radius: the directional derivative of a linear loss along a random
+    weight direction against central differences of the FP64 iteration (step 1e-4: truncation below
+    1e-6 of the derivative, float32 roundings of 3 steps below 1e-5)."""
+    rng = np.random.default_rng(5)
+    V = rng.random((2, T, H, W)).astype(np.float32)
+    c = rng.normal(size=(T, H, W)).astype(np.float32)
+    w = np.array([0.8, -0.5], dtype=np.float32)
+    r = (1, 6, 6)
+    with sf.PowerIteration(2, T, H, W) as h:
+        h.power_iterate(torch.from_numpy(V).cuda(), w, 0.1, r, iters=3, record_every=2)
+        gw, gb = h.backward(torch.from_numpy(c).cuda(), r)
+    d = np.array([0.6, 0.8, -0.5])                   # direction in (w0, w1, b)
+
+    def loss(t):
+        f = oracle.combine(V.astype(np.float64), w.astype(np.float64) + t * d[:2], 0.1 + t * d[2])
+        x, _ = oracle.power_filter(f, f, 0.1, 1.0, r, np.ones(f.shape), 3)
+        return float((x * c).sum())
+
+    num = (loss(1e-4) - loss(-1e-4)) / 2e-4
+    scale = float(np.abs(np.append(gw, gb)).max())
+    assert abs(gw[0] * d[0] + gw[1] * d[1] + gb * d[2] - num) <= 1e-4 * scale
