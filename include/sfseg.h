@@ -140,14 +140,14 @@ int sfseg_apply(sfseg_handle* h, const sfseg_neighborhood* nb, const float* x, f
  * M_ij = u_i u_j exp(-alpha (f_i - f_j)^2) G_ij on the same box, Gaussian and zero padding as
  * sfseg_apply (the 1/alpha matches A = M/alpha of Eq. 7, so both operators have comparable
  * eigenvalues; eigenvectors do not depend on it).  Computed without forming M, through the
- * series exp(-alpha (f_i - f_j)^2) = e^{-alpha f_i^2} e^{-alpha f_j^2} sum_n (2 alpha f_i f_j)^n / n!,
- * whose terms are separable: three terms per pass of the TMA stencil.  Shared maps only
+ * series exp(-alpha (f_i - f_j)^2) = e^{-alpha g_i^2} e^{-alpha g_j^2} sum_n (2 alpha g_i g_j)^n / n!
+ * in g = f - c, whose terms are separable: three terms per pass of the TMA stencil.  Shared maps only
  * (UNSUPPORTED after sfseg_set_features_sf), the radii with a TMA kernel only (UNSUPPORTED
- * otherwise), FP32 storage.
- *   n_terms   the number of series terms, 1..120; 0 chooses the smallest count whose tail
- *             bound x^(N+1)/(N+1)! e^x, x = 2 alpha max(f)^2, is below 2^-24 relative to the sum
- *             (this reads max f: the call synchronises), or returns UNSUPPORTED when 120 terms
- *             do not reach it.
+ * otherwise), FP32 storage.  Allocates three more float32 volumes on first use.
+ *   n_terms   the number of terms of the series in f (c = 0), 1..120; 0 takes c in the middle of f's
+ *             range and the smallest count whose tail bound x^(N+1)/(N+1)! e^x, x = 2 alpha max(g)^2,
+ *             is below 2^-24 relative to the sum (this reads f's range: the call synchronises), or
+ *             returns UNSUPPORTED when 120 terms of the series in f do not reach that.
  *   x, y      device [T][H][W] float32 (may not alias).
  * Errors: INVALID_ARG, SHAPE, STATE (no features), UNSUPPORTED, OOM, CUDA. */
 int sfseg_apply_exact(sfseg_handle* h, const sfseg_neighborhood* nb, int n_terms, const float* x,

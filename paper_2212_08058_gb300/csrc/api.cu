@@ -109,7 +109,8 @@ struct sfseg_handle {
     float* adjw[3] = {nullptr, nullptr, nullptr};   // TMA-path adjoint workspace (Q_g, v_g, v_g)
     std::vector<float*> seg;
     std::vector<float*> qxs;   // TMA path: Q_x of each step of the segment being reversed
-    float* exv = nullptr;      // the exact kernel's term input (internal layout)
+    // the exact kernel (internal layout): the term input, g = f - c and A = u e^{-alpha g^2}
+    float *exv = nullptr, *exg = nullptr, *exa = nullptr;
     double* dots = nullptr;
     int dots_cap = 0;
     // optional CUDA-event timing of the iteration kernels
@@ -349,6 +350,8 @@ int sfseg_destroy(sfseg_handle* h) {
     for (float* p : h->seg) cudaFree(p);
     for (float* p : h->qxs) cudaFree(p);
     cudaFree(h->exv);
+    cudaFree(h->exg);
+    cudaFree(h->exa);
     cudaFree(h->dots);
     for (sfseg_handle* c : h->lvl) sfseg_destroy(c);
     for (float* p : h->lvl_f) cudaFree(p);
@@ -622,55 +625,63 @@ int sfseg_apply(sfseg_handle* h, const sfseg_neighborhood* nb, const float* x, f
 namespace {
 constexpr int kExactMaxTerms = 120;   // 40 launches of three terms
 
-// The series length N + 1: n_terms if given, else the smallest N whose tail bound
-// x^(N+1)/(N+1)! e^x (x = 2 alpha max(f)^2, relative to the series' sum >= 1) is below 2^-24.
-int exact_terms(sfseg_handle* h, int n_terms, cudaStream_t s, int* terms_out) {
+// The smallest number of terms, N + 1, whose tail bound x^(N+1)/(N+1)! e^x (x = 2 alpha max(g)^2),
+// relative to the series' sum >= e^-lo, is below 2^-24; 0 if kExactMaxTerms do not reach it.
+int series_length(double x, double lo) {
+    double tail = x * std::exp(x + lo);   // N = 0
+    for (int n = 1; n <= kExactMaxTerms; ++n) {
+        if (tail <= std::ldexp(1.0, -24)) return n;
+        tail *= x / (n + 1);
+    }
+    return 0;
+}
+
+// The number of series terms and the centre c of g = f - c.  n_terms > 0 is the caller's choice of
+// the series in f (c = 0).  Otherwise c is the middle of f's range, which halves max |g| for f from 0:
+// a quarter of x, and about half the terms.  A call whose series in f would be too long is refused
+// whatever the centred one needs.
+int exact_terms(sfseg_handle* h, int n_terms, cudaStream_t s, int* terms_out, float* center) {
     if (n_terms < 0 || n_terms > kExactMaxTerms)
-        return fail(SFSEG_ERR_INVALID_ARG, "n_terms must be in [0, 120] (0: chosen from alpha and max f)");
+        return fail(SFSEG_ERR_INVALID_ARG, "n_terms must be in [0, 120] (0: chosen from alpha and f's range)");
+    *center = 0.f;
     if (n_terms > 0) {
         *terms_out = n_terms;
         return SFSEG_OK;
     }
-    unsigned* key = reinterpret_cast<unsigned*>(h->scratch + kScrMaxKey);
-    SFSEG_CUDA(cudaMemsetAsync(key, 0, sizeof(unsigned), s));
-    launch_max_key(h->f32, h->NP, key, s);
+    unsigned* keys = reinterpret_cast<unsigned*>(h->scratch + kScrMaxKey);   // max f, max -f
+    SFSEG_CUDA(cudaMemsetAsync(keys, 0, 2 * sizeof(unsigned), s));
+    launch_exact_range(h->f32, h->g, keys, s);
     SFSEG_LAUNCHED();
-    unsigned k = 0;
-    SFSEG_CUDA(cudaMemcpyAsync(&k, key, sizeof(k), cudaMemcpyDeviceToHost, s));
+    unsigned k[2] = {0, 0};
+    SFSEG_CUDA(cudaMemcpyAsync(k, keys, sizeof(k), cudaMemcpyDeviceToHost, s));
     SFSEG_CUDA(cudaStreamSynchronize(s));
-    uint32_t b = (k & 0x80000000u) ? (k & 0x7fffffffu) : ~k;
-    float fmax;
-    std::memcpy(&fmax, &b, sizeof(fmax));
-    const double x = 2.0 * h->alpha * (double)fmax * fmax;
-    double tail = x * std::exp(x);   // x^(N+1)/(N+1)! e^x for N = 0
-    for (int n = 1; n <= kExactMaxTerms; ++n) {
-        if (tail <= std::ldexp(1.0, -24)) {
-            *terms_out = n;
-            return SFSEG_OK;
-        }
-        tail *= x / (n + 1);
+    float v[2];
+    for (int i = 0; i < 2; ++i) {
+        const uint32_t b = (k[i] & 0x80000000u) ? (k[i] & 0x7fffffffu) : ~k[i];
+        std::memcpy(&v[i], &b, sizeof(float));
     }
-    return fail(SFSEG_ERR_UNSUPPORTED, "alpha * max(f)^2 too large for the series form of the exact kernel");
+    const double fmax = v[0], fmin = -(double)v[1];
+    if (!series_length(2.0 * h->alpha * fmax * fmax, 0.0))
+        return fail(SFSEG_ERR_UNSUPPORTED, "alpha * max(f)^2 too large for the series form of the exact kernel");
+    *center = (float)(0.5 * (fmax + fmin));
+    const double r = std::max(fmax - *center, *center - fmin), x = 2.0 * h->alpha * r * r;
+    *terms_out = std::max(series_length(x, x), 1);   // products g_i g_j may be negative: sum >= e^-x
+    return SFSEG_OK;
 }
 
-// y = (1/alpha) M x~ s (s = 1/sqrt(*acc_in), or 1), internal layout; acc_out += ||y||^2.
-int exact_apply(sfseg_handle* h, const Taps& tp, int terms, const float* xt, const double* acc_in, float* y,
-                double* acc_out, cudaStream_t s) {
+// S = s sum_n c_n g^n G*(g^n w) for w in exv (which it uses up), s = 1/sqrt(*acc) (or 1).
+int exact_series(sfseg_handle* h, const Taps& tp, int terms, const double* acc, float* S, cudaStream_t s) {
     const double a = h->alpha;
     std::vector<double> c((size_t)terms + 2, 0.0);
     c[0] = 1.0;
     for (int n = 1; n < terms; ++n) c[n] = c[n - 1] * 2.0 * a / n;
     const int groups = (terms + 2) / 3;
     for (int j = 0; j < groups; ++j) {
-        launch_exact_prep(xt, acc_in, h->f32, (float)a, (float)h->p, j, h->g, h->exv, h->flags, s);
-        SFSEG_LAUNCHED();
+        if (j > 0) launch_exact_next(h->exg, h->g, h->exv, s);
         ExactTerm ex;
         ex.j = j;
-        ex.last = j == groups - 1;
         for (int i = 0; i < 3; ++i) ex.c[i] = 3 * j + i < terms ? (float)c[3 * j + i] : 0.f;
-        ex.alpha = (float)a;
-        if (!launch_exact_term_fast(h->exv, y, h->f32, h->g, tp, (float)(1.0 / a), (float)h->p, ex,
-                                    ex.last ? acc_out : nullptr, h->flags, s))
+        if (!launch_exact_term_fast(h->exv, S, h->exg, h->g, tp, ex, acc, h->flags, s))
             return fail(SFSEG_ERR_CUDA, "the TMA stencil could not be launched");
         SFSEG_LAUNCHED();
     }
@@ -682,7 +693,8 @@ int exact_checks(sfseg_handle* h, const Taps& tp) {
     if (h->sep) return fail(SFSEG_ERR_UNSUPPORTED, "the exact kernel is for shared maps (S = F)");
     if (!fast_iterate_supported(tp))
         return fail(SFSEG_ERR_UNSUPPORTED, "the exact kernel runs on the radii with a TMA kernel only");
-    if (!h->exv) SFSEG_CUDA(dalloc(&h->exv, (size_t)h->NP));
+    for (float** q : {&h->exv, &h->exg, &h->exa})
+        if (!*q) SFSEG_CUDA(dalloc(q, (size_t)h->NP));
     return SFSEG_OK;
 }
 }  // namespace
@@ -697,13 +709,14 @@ int sfseg_apply_exact(sfseg_handle* h, const sfseg_neighborhood* nb, int n_terms
     if (int rc = exact_checks(h, tp)) return rc;
     cudaStream_t s = (cudaStream_t)stream;
     int terms = 0;
-    if (int rc = exact_terms(h, n_terms, s, &terms)) return rc;
-    float* xt = (float*)h->vbuf[0];
-    float* yt = (float*)h->vbuf[1];
-    launch_exact_in(x, h->g, xt, nullptr, s);
+    float center = 0.f;
+    if (int rc = exact_terms(h, n_terms, s, &terms, &center)) return rc;
+    float* S = (float*)h->vbuf[0];
+    launch_exact_setup(h->f32, center, (float)h->alpha, (float)h->p, h->g, h->exg, h->exa, s);
+    launch_exact_in(x, h->exa, h->g, h->exv, nullptr, s);
     SFSEG_LAUNCHED();
-    if (int rc = exact_apply(h, tp, terms, xt, nullptr, yt, nullptr, s)) return rc;
-    launch_exact_out(yt, nullptr, h->g, y, h->flags, s);
+    if (int rc = exact_series(h, tp, terms, nullptr, S, s)) return rc;
+    launch_exact_out(S, h->exa, (float)(1.0 / h->alpha), h->g, y, nullptr, s);
     SFSEG_LAUNCHED();
     return SFSEG_OK;
 }
@@ -720,16 +733,28 @@ int sfseg_power_iterate_exact(sfseg_handle* h, const sfseg_neighborhood* nb, int
     if (int rc = exact_checks(h, tp)) return rc;
     cudaStream_t s = (cudaStream_t)stream;
     int terms = 0;
-    if (int rc = exact_terms(h, n_terms, s, &terms)) return rc;
+    float center = 0.f;
+    if (int rc = exact_terms(h, n_terms, s, &terms, &center)) return rc;
     if (int rc = ensure_acc(&h->acc, &h->acc_cap, iters + 2)) return rc;
     double* acc = h->acc;
     SFSEG_CUDA(cudaMemsetAsync(acc, 0, sizeof(double) * (iters + 1), s));
-    float* buf[2] = {(float*)h->vbuf[0], (float*)h->vbuf[1]};
-    launch_exact_in(init == SFSEG_INIT_USER ? x_inout : nullptr, h->g, buf[0], acc, s);
-    SFSEG_LAUNCHED();
-    for (int k = 0; k < iters; ++k)
-        if (int rc = exact_apply(h, tp, terms, buf[k & 1], acc + k, buf[(k + 1) & 1], acc + k + 1, s)) return rc;
-    launch_exact_out(buf[iters & 1], acc + iters, h->g, x_inout, h->flags, s);
+    const float inv_alpha = (float)(1.0 / h->alpha);
+    float* S = (float*)h->vbuf[0];
+    const float* x_user = init == SFSEG_INIT_USER ? x_inout : nullptr;
+    if (iters == 0) {   // x0 itself, normalised
+        if (!x_user) launch_fill(x_inout, h->N, 1.f, s);
+        launch_sumsq(x_inout, h->N, acc, s);
+    } else {
+        launch_exact_setup(h->f32, center, (float)h->alpha, (float)h->p, h->g, h->exg, h->exa, s);
+        launch_exact_in(x_user, h->exa, h->g, h->exv, acc, s);
+        SFSEG_LAUNCHED();
+        for (int k = 0; k < iters; ++k) {
+            if (int rc = exact_series(h, tp, terms, acc + k, S, s)) return rc;
+            if (k + 1 < iters) launch_exact_mid(S, h->exa, inv_alpha, h->g, h->exv, acc + k + 1, s);
+            else launch_exact_out(S, h->exa, inv_alpha, h->g, x_inout, acc + iters, s);
+        }
+    }
+    launch_scale_inv_norm(x_inout, h->N, acc + iters, h->flags, s);
     SFSEG_LAUNCHED();
     if (norms_out) {
         std::vector<double> a((size_t)iters + 1);

@@ -152,10 +152,9 @@ struct Params {
     double* acc_out;
     int* flags;
     void* out;        // OUT_X: x~ (caller layout)
-    // MODE 7 only: term j of the exact kernel's series (see below)
-    int exj, exlast;
+    // MODE 7 only: term group j of the exact kernel's series (see below)
+    int exj;
     float exc[3];     // c_{3j}, c_{3j+1}, c_{3j+2}
-    float ex_alpha;
     unsigned* maxkey; // MODE 8: atomicMax of the order key of the largest output
 };
 
@@ -202,12 +201,11 @@ __device__ __forceinline__ bool run_of(const Params& P, int s, Run& r) {
 // voxels to acc_out, with V_k = u x~_k the second input (so that <x_k, A z> = s_k sum V_k B needs
 // no division by u).  MODE 6 is the step (MODE 0, the state to out) that also stores s Q to out2:
 // the adjoint's recomputation and Q-pass share the filtering of V_k.  MODE 7 serves the exact
-// (Eq. 1) kernel, exp(-a (f_i - f_j)^2) = e^{-a f_i^2} e^{-a f_j^2} sum_n c_n f_i^n f_j^n with
-// c_n = (2a)^n / n!: for the input v = f^{3j} w, its three filtered signals are the series
-// terms n = 3j (G*v), 3j + 1 (G*(f v)) and 3j + 2 (G*(f^2 v)); it adds
-// t = f^{3j} (c_{3j} G*v + f (c_{3j+1} G*(f v) + f c_{3j+2} G*(f^2 v))) to out (writes it when
-// j = 0), and on the last term stores y = u e^{-a f^2} / a * (sum of the terms) and adds |y|^2 to
-// acc_out.  All in the internal layout.  MODE 8 is the step (MODE 0) that also takes the
+// (Eq. 1) kernel, exp(-a (f_i - f_j)^2) = e^{-a g_i^2} e^{-a g_j^2} sum_n c_n g_i^n g_j^n with
+// c_n = (2a)^n / n! and g = f - c for any constant c: with g in f's place and the input v = g^{3j} w,
+// its three filtered signals are the series terms n = 3j (G*v), 3j + 1 (G*(g v)) and 3j + 2
+// (G*(g^2 v)); it adds t = s g^{3j} (c_{3j} G*v + g (c_{3j+1} G*(g v) + g c_{3j+2} G*(g^2 v))) to out
+// (writes it when j = 0).  All in the internal layout.  MODE 8 is the step (MODE 0) that also takes the
 // largest of its outputs and adds it to P.maxkey (atomicMax of the order key, one per CTA): the
 // maximum a soft-binarisation step (Alg. 1 step 3) scales by, without a pass of its own.
 template <int RT, int RH, int RW, typename TS, typename TVO, bool OUT_X, bool SEP, int MODE>
@@ -518,14 +516,8 @@ iter_stream(const __grid_constant__ Maps M, const __grid_constant__ Params P) {
                             const float2 f3 = mul2(fv, mul2(fv, fv));
                             for (int i3 = 0; i3 < P.exj; ++i3) F = mul2(F, f3);
                             const float2 inner = fma2(mul2(fv, f2(P.exc[2])), y[1][m], mul2(f2(P.exc[1]), y[2][m]));
-                            outv[m] = mul2(F, fma2(fv, inner, mul2(f2(P.exc[0]), y[0][m])));
+                            outv[m] = mul2(mul2(s2, F), fma2(fv, inner, mul2(f2(P.exc[0]), y[0][m])));
                             if (P.exj > 0) outv[m] = __fadd2_rn(outv[m], so[m]);   // the terms so far
-                            if (P.exlast) {
-                                const float2 a = make_float2(u.x * expf(-P.ex_alpha * fv.x * fv.x) * P.inv_alpha,
-                                                             u.y * expf(-P.ex_alpha * fv.y * fv.y) * P.inv_alpha);
-                                outv[m] = mul2(a, outv[m]);
-                                part = fma2(outv[m], outv[m], part);
-                            }
                         } else if constexpr (MODE == 0 || MODE == 4 || MODE == 6 || MODE == 8) {
                             float2 B = fma2(ee, y[0][m], make_float2(-y[1][m].x, -y[1][m].y));
                             B = fma2(mul2(f2(2.f), fv), y[2][m], B);
@@ -635,9 +627,7 @@ static bool launch_t(const StepArgs& a) {
     fill(P.gh, RH, a.tp.gh, a.tp.rh);
     fill(P.gw, RW, a.tp.gw, a.tp.rw);
     P.exj = a.ex ? a.ex->j : 0;
-    P.exlast = a.ex ? a.ex->last : 0;
     for (int i = 0; i < 3; ++i) P.exc[i] = a.ex ? a.ex->c[i] : 0.f;
-    P.ex_alpha = a.ex ? a.ex->alpha : 0.f;
     P.maxkey = a.maxkey;
     P.tx = (g.W + TW - 1) / TW;
     P.tiles = P.tx * ((g.H + TH - 1) / TH);

@@ -91,10 +91,9 @@ struct Params {
     const float* s;   // separate unary map S_m (SEP kernels), or the state V_k (MODE 5); float32,
                       // internal pitch
     void* out2;       // second output: the record x~ (MODE 4) or Q (MODEs 5 and 6)
-    // MODE 7 only: term j of the exact kernel's series (see below)
-    int exj, exlast;
+    // MODE 7 only: term group j of the exact kernel's series
+    int exj;
     float exc[3];     // c_{3j}, c_{3j+1}, c_{3j+2}
-    float ex_alpha;
     unsigned* maxkey; // MODE 8: atomicMax of the order key of the largest output
 };
 
@@ -306,7 +305,7 @@ iter_tile(const __grid_constant__ CUtensorMap mv, const __grid_constant__ CUtens
                     const float2 f3 = mul2(fv, mul2(fv, fv));
                     for (int i = 0; i < P.exj; ++i) F = mul2(F, f3);
                     const float2 inner = fma2(mul2(fv, f2(P.exc[2])), y[1][m], mul2(f2(P.exc[1]), y[2][m]));
-                    outv[m] = mul2(F, fma2(fv, inner, mul2(f2(P.exc[0]), y[0][m])));
+                    outv[m] = mul2(mul2(s2, F), fma2(fv, inner, mul2(f2(P.exc[0]), y[0][m])));
                 } else if constexpr (MODE == 0 || MODE == 4 || MODE == 6 || MODE == 8) {
                     float2 B = fma2(e, y[0][m], make_float2(-y[1][m].x, -y[1][m].y));
                     B = fma2(mul2(f2(2.f), fv), y[2][m], B);
@@ -351,17 +350,6 @@ iter_tile(const __grid_constant__ CUtensorMap mv, const __grid_constant__ CUtens
                         for (int m = 0; m < 4; ++m) {
                             if (wbase + 2 * m + 1 < g.W) outv[m] = __fadd2_rn(outv[m], ld_pair(o + 2 * m));
                             else if (wbase + 2 * m < g.W) outv[m].x += o[2 * m];
-                        }
-                    }
-                    if (P.exlast) {
-#pragma unroll
-                        for (int m = 0; m < 4; ++m) {
-                            const float2 fv = fo[m];
-                            const float2 a = make_float2(
-                                unary_pow_fast(fv.x, P.p) * expf(-P.ex_alpha * fv.x * fv.x) * P.inv_alpha,
-                                unary_pow_fast(fv.y, P.p) * expf(-P.ex_alpha * fv.y * fv.y) * P.inv_alpha);
-                            outv[m] = mul2(a, outv[m]);
-                            part = fma2(outv[m], outv[m], part);
                         }
                     }
                     st_pairs(o, outv, wbase, g.W);
@@ -496,9 +484,7 @@ static bool launch_t(const StepArgs& a) {
     P.s = a.s32;
     P.out2 = a.out2;
     P.exj = a.ex ? a.ex->j : 0;
-    P.exlast = a.ex ? a.ex->last : 0;
     for (int i = 0; i < 3; ++i) P.exc[i] = a.ex ? a.ex->c[i] : 0.f;
-    P.ex_alpha = a.ex ? a.ex->alpha : 0.f;
     P.maxkey = a.maxkey;
     const int tx = (g.W + TW - 1) / TW, ty = (g.H + TH - 1) / TH;
     P.tchunk = pick_chunk(g.T, tx * ty, slots_per_sm * num_sms(), RT);

@@ -1,61 +1,158 @@
 // kernels_exact.cu -- the element-wise parts of the exact (Eq. 1) kernel's operator, the
 // diagnostic of the first-order approximation (Sec. 4.3): M_ij = u_i u_j exp(-a (f_i - f_j)^2) G_ij
-// written as the series e^{-a f_i^2} e^{-a f_j^2} sum_n c_n f_i^n f_j^n, c_n = (2a)^n / n!, whose
-// terms are separable and go through the TMA stencil three at a time (kernels_fast.cu, mode 7).
-// Here: the iterate into the internal layout, the input v = f^{3j} w of term group j with
-// w = s u e^{-a f^2} x~, and the result back into the caller's layout.
+// written with g = f - c as the series e^{-a g_i^2} e^{-a g_j^2} sum_n c_n g_i^n g_j^n,
+// c_n = (2a)^n / n!, whose terms are separable and go through the TMA kernels three at a time
+// (iter_stream.cuh, mode 7).  With A = u e^{-a g^2} a step is: w = A x~, S = s sum_n c_n g^n G*(g^n w),
+// the next x~ = A S / a.  The norm s = 1/||x~|| is summed by the pass that forms w and applied by the
+// filtering (the operator is linear), so no pass waits for it.
+//
+// c = 0 is the series in f itself.  The middle of f's range halves max |g|, and the terms needed
+// follow x = 2 a max(g)^2: 9 instead of 16 for f in [0, 1] at a = 1, three filterings a step instead of
+// six.  These passes move 12 bytes per voxel, four columns per thread (rows start 128-byte aligned);
+// forming each group's input from x~ with the power and the exponential took 12 bytes and, with the
+// norm's FP64 in every thread, 28.6 us for 3.3M voxels.  Five steps at 32x240x427, (2,7,7), the call:
+// 1449 us with the series in f, 659 us now.
 #include "launch.h"
+#include "order_key.cuh"
 #include "voxels.cuh"
 
 namespace sfseg {
 
-// x~ (internal) = the caller's x, or 1 everywhere (x_user null); acc += ||x~||^2.
-__global__ void exact_in_kernel(const float* x_user, Geom g, float* xt, double* acc) {
-    float part = 0.f;
-    for_each_voxel(g, [&](int64_t i, int64_t j) {
-        const float v = x_user ? x_user[i] : 1.f;
-        xt[j] = v;
-        part += v * v;
-    });
+namespace {
+
+// f4(j) for the groups of four columns of every internal row, f1(i, j) for the ragged ends (i the
+// caller-layout index, j the internal one).
+template <typename F4, typename F1>
+__device__ __forceinline__ void for_each_quad(const Geom& g, F4&& f4, F1&& f1) {
+    const int64_t rows = (int64_t)g.T * g.H;
+    const int w4 = g.W / 4;
+    for (int64_t row = blockIdx.x; row < rows; row += gridDim.x) {
+        const int64_t j0 = row * g.pitch, i0 = row * g.W;
+        for (int c = threadIdx.x; c < w4; c += blockDim.x) f4(j0 + 4 * c);
+        for (int w = 4 * w4 + threadIdx.x; w < g.W; w += blockDim.x) f1(i0 + w, j0 + w);
+    }
+}
+__device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
+__device__ __forceinline__ void st4(float* p, float4 v) { *reinterpret_cast<float4*>(p) = v; }
+
+RowLaunch quad_launch(const Geom& g, int per_sm) {
+    const int64_t rows = (int64_t)g.T * g.H, cap = (int64_t)per_sm * num_sms();
+    const int w4 = (g.W + 3) / 4;
+    return {(int)(rows < cap ? rows : cap), w4 >= 128 ? 128 : (w4 + 31) / 32 * 32};
+}
+
+__device__ __forceinline__ void add_sum(float part, double* acc) {
     const double b = block_sum((double)part);
     if (threadIdx.x == 0 && acc) atomicAdd(acc, b);
 }
 
-// v = f^{3j} s u e^{-a f^2} x~, s = 1/sqrt(*acc) (1 if acc is null).
-__global__ void exact_prep_kernel(const float* xt, const double* acc, const float* f, float alpha, float p, int jt,
-                                  Geom g, float* v, int* flags) {
-    const float s = block_inv_norm(acc, flags);
+}  // namespace
+
+__global__ void exact_range_kernel(const float* f, Geom g, unsigned* keys) {
+    unsigned hi = 0u, lo = 0u;
     for_each_voxel(g, [&](int64_t, int64_t j) {
-        const float fv = f[j];
-        const float f3 = fv * fv * fv;
-        float F = 1.f;
-        for (int i = 0; i < jt; ++i) F *= f3;
-        v[j] = F * (s * unary_pow_fast(fv, p) * expf(-alpha * fv * fv) * xt[j]);
+        hi = max(hi, order_key(f[j]));
+        lo = max(lo, order_key(-f[j]));
+    });
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    lo = __reduce_max_sync(0xffffffffu, lo);
+    if ((threadIdx.x & 31) == 0) {
+        atomicMax(keys, hi);
+        atomicMax(keys + 1, lo);
+    }
+}
+
+__global__ void exact_setup_kernel(const float* f, float center, float alpha, float p, Geom g, float* gf, float* A) {
+    for_each_voxel(g, [&](int64_t, int64_t j) {
+        const float fv = f[j], gv = fv - center;
+        gf[j] = gv;
+        A[j] = unary_pow_fast(fv, p) * expf(-alpha * gv * gv);
     });
 }
 
-// The caller's x = s y (y internal), s = 1/sqrt(*acc) (1 if acc is null).
-__global__ void exact_out_kernel(const float* y, const double* acc, Geom g, float* x_user, int* flags) {
-    const float s = block_inv_norm(acc, flags);
-    for_each_voxel(g, [&](int64_t i, int64_t j) { x_user[i] = s * y[j]; });
+__global__ void exact_in_kernel(const float* x_user, const float* A, Geom g, float* w, double* acc) {
+    float part = 0.f;
+    for_each_voxel(g, [&](int64_t i, int64_t j) {
+        const float v = x_user ? x_user[i] : 1.f;
+        w[j] = A[j] * v;
+        part += v * v;
+    });
+    add_sum(part, acc);
 }
 
-void launch_exact_in(const float* x_user, Geom g, float* xt, double* acc, cudaStream_t s) {
-    const RowLaunch rl = row_launch(g, num_sms());
-    exact_in_kernel<<<rl.blocks, rl.threads, 0, s>>>(x_user, g, xt, acc);
+__global__ void exact_mid_kernel(const float* S, const float* A, float inv_alpha, Geom g, float* w, double* acc) {
+    float part = 0.f;
+    auto one = [&](float s, float a) {
+        const float x = a * s * inv_alpha;
+        part += x * x;
+        return a * x;
+    };
+    for_each_quad(
+        g,
+        [&](int64_t j) {
+            const float4 s = ld4(S + j), a = ld4(A + j);
+            st4(w + j, make_float4(one(s.x, a.x), one(s.y, a.y), one(s.z, a.z), one(s.w, a.w)));
+        },
+        [&](int64_t, int64_t j) { w[j] = one(S[j], A[j]); });
+    add_sum(part, acc);
+}
+
+__global__ void exact_next_kernel(const float* gf, Geom g, float* v) {
+    for_each_quad(
+        g,
+        [&](int64_t j) {
+            const float4 a = ld4(gf + j), x = ld4(v + j);
+            st4(v + j, make_float4(a.x * a.x * a.x * x.x, a.y * a.y * a.y * x.y, a.z * a.z * a.z * x.z,
+                                   a.w * a.w * a.w * x.w));
+        },
+        [&](int64_t, int64_t j) { v[j] *= gf[j] * gf[j] * gf[j]; });
+}
+
+__global__ void exact_out_kernel(const float* S, const float* A, float inv_alpha, Geom g, float* x_user, double* acc) {
+    float part = 0.f;
+    for_each_voxel(g, [&](int64_t i, int64_t j) {
+        const float x = A[j] * S[j] * inv_alpha;
+        x_user[i] = x;
+        part += x * x;
+    });
+    add_sum(part, acc);
+}
+
+void launch_exact_range(const float* f32, Geom g, unsigned* keys, cudaStream_t s) {
+    const RowLaunch rl = row_launch(g, num_sms(), 8);
+    exact_range_kernel<<<rl.blocks, rl.threads, 0, s>>>(f32, g, keys);
     count_launches(1);
 }
 
-void launch_exact_prep(const float* xt, const double* acc, const float* f32, float alpha, float p, int jt, Geom g,
-                       float* v, int* flags, cudaStream_t s) {
+void launch_exact_setup(const float* f32, float center, float alpha, float p, Geom g, float* gf, float* A,
+                        cudaStream_t s) {
     const RowLaunch rl = row_launch(g, num_sms());
-    exact_prep_kernel<<<rl.blocks, rl.threads, 0, s>>>(xt, acc, f32, alpha, p, jt, g, v, flags);
+    exact_setup_kernel<<<rl.blocks, rl.threads, 0, s>>>(f32, center, alpha, p, g, gf, A);
     count_launches(1);
 }
 
-void launch_exact_out(const float* y, const double* acc, Geom g, float* x_user, int* flags, cudaStream_t s) {
-    const RowLaunch rl = row_launch(g, num_sms());
-    exact_out_kernel<<<rl.blocks, rl.threads, 0, s>>>(y, acc, g, x_user, flags);
+void launch_exact_in(const float* x_user, const float* A, Geom g, float* w, double* acc, cudaStream_t s) {
+    const RowLaunch rl = row_launch(g, num_sms(), 8);
+    exact_in_kernel<<<rl.blocks, rl.threads, 0, s>>>(x_user, A, g, w, acc);
+    count_launches(1);
+}
+
+void launch_exact_mid(const float* S, const float* A, float inv_alpha, Geom g, float* w, double* acc, cudaStream_t s) {
+    const RowLaunch rl = quad_launch(g, 16);
+    exact_mid_kernel<<<rl.blocks, rl.threads, 0, s>>>(S, A, inv_alpha, g, w, acc);
+    count_launches(1);
+}
+
+void launch_exact_next(const float* gf, Geom g, float* v, cudaStream_t s) {
+    const RowLaunch rl = quad_launch(g, 16);
+    exact_next_kernel<<<rl.blocks, rl.threads, 0, s>>>(gf, g, v);
+    count_launches(1);
+}
+
+void launch_exact_out(const float* S, const float* A, float inv_alpha, Geom g, float* x_user, double* acc,
+                      cudaStream_t s) {
+    const RowLaunch rl = row_launch(g, num_sms(), 8);
+    exact_out_kernel<<<rl.blocks, rl.threads, 0, s>>>(S, A, inv_alpha, g, x_user, acc);
     count_launches(1);
 }
 

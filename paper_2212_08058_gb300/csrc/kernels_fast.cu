@@ -165,9 +165,9 @@ bool launch_step_q_fast(const float* vin, float* vout, float* Q, const float* f,
     return run(a);
 }
 
-bool launch_exact_term_fast(const float* v, float* y, const float* f, const Geom& g, const Taps& tp, float inv_alpha,
-                            float p, const ExactTerm& ex, double* acc_out, int* flags, cudaStream_t s) {
-    StepArgs a = args(kExactTerm, v, y, f, g, tp, inv_alpha, p, nullptr, acc_out, flags, s);
+bool launch_exact_term_fast(const float* v, float* y, const float* gf, const Geom& g, const Taps& tp,
+                            const ExactTerm& ex, const double* acc_in, int* flags, cudaStream_t s) {
+    StepArgs a = args(kExactTerm, v, y, gf, g, tp, 1.f, 1.f, acc_in, nullptr, flags, s);
     a.ex = &ex;
     return run(a);
 }

@@ -362,6 +362,18 @@ void launch_to_bf16(const float* a, __nv_bfloat16* b, int64_t n, cudaStream_t s)
     to_bf16_kernel<<<blocks, 256, 0, s>>>(a, b, n); count_launches(1);
 }
 
+// x = v over n elements.
+__global__ void fill_kernel(float* x, int64_t n, float v) {
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+        x[i] = v;
+}
+
+void launch_fill(float* x, int64_t n, float v, cudaStream_t s) {
+    const int64_t b = (n + 255) / 256;
+    fill_kernel<<<(int)(b < 1024 ? b : 1024), 256, 0, s>>>(x, n, v);
+    count_launches(1);
+}
+
 // ------------------------------------------------------------------------- reductions
 __global__ void scale_inv_norm_kernel(float* x, int64_t n, bool vec, const double* acc, int* flags) {
     const float s = block_inv_norm(acc, flags);

@@ -69,27 +69,30 @@ bool launch_iterate_fast_ckpt(const float* vin, void* out, bool out_x, const flo
 bool launch_filter_fast(const float* vin, float* out, const float* f, const Geom& g, const Taps& tp, float inv_alpha,
                         float p, const double* acc_in, int* flags, cudaStream_t s);
 
-// One term j of the exact (Eq. 1) kernel's series on the TMA kernel (kernels_fast.cu, mode 7):
-// for the input v = f^{3j} w (internal layout), adds the terms n = 3j, 3j+1, 3j+2 of
-// sum_n c_n f^n G*(f^n w) to y (writes them when j = 0); on the last term multiplies the sum by
-// u e^{-alpha f^2} / alpha and adds ||y||^2 to *acc_out (nullable).  Returns false for a radius
-// without a compiled kernel.
+// One term group j of the exact (Eq. 1) kernel's series on the TMA kernels (mode 7 at iter_stream):
+// for the input v = g^{3j} w (internal layout), adds the terms n = 3j, 3j+1, 3j+2 of
+// s sum_n c_n g^n G*(g^n w) to y (writes them when j = 0), s = 1/sqrt(*acc_in) (or 1).  Returns false
+// for a radius without a compiled kernel.
 struct ExactTerm {
-    int j, last;
+    int j;
     float c[3];     // c_{3j}, c_{3j+1}, c_{3j+2}, c_n = (2 alpha)^n / n! (0 beyond the last term)
-    float alpha;
 };
-bool launch_exact_term_fast(const float* v, float* y, const float* f, const Geom& g, const Taps& tp, float inv_alpha,
-                            float p, const ExactTerm& ex, double* acc_out, int* flags, cudaStream_t s);
+bool launch_exact_term_fast(const float* v, float* y, const float* gf, const Geom& g, const Taps& tp,
+                            const ExactTerm& ex, const double* acc_in, int* flags, cudaStream_t s);
 
-// The exact kernel's element-wise parts (kernels_exact.cu, internal layout unless noted): x~ from
-// the caller's x (or 1 everywhere for a null x_user) with acc += ||x~||^2 (nullable); the input
-// of term group j, v = f^{3j} s u e^{-alpha f^2} x~ with s = 1/sqrt(*acc) (or 1); and the
-// caller's x = s y.
-void launch_exact_in(const float* x_user, Geom g, float* xt, double* acc, cudaStream_t s);
-void launch_exact_prep(const float* xt, const double* acc, const float* f32, float alpha, float p, int jt, Geom g,
-                       float* v, int* flags, cudaStream_t s);
-void launch_exact_out(const float* y, const double* acc, Geom g, float* x_user, int* flags, cudaStream_t s);
+// The exact kernel's element-wise parts (kernels_exact.cu, internal layout unless noted).  Keys of
+// max f and of max(-f) over the voxels (order_key.cuh; zero both first); g = f - c and
+// A = u e^{-alpha g^2}; the first step's w = A x0 (x0 the caller's, or 1) with acc += ||x0||^2; the next
+// step's w = A x~ with x~ = A S / alpha and acc += ||x~||^2; v = g^3 v in place; and the caller's
+// x~ = A S / alpha with acc += ||x~||^2.  acc is nullable.
+void launch_exact_range(const float* f32, Geom g, unsigned* keys, cudaStream_t s);
+void launch_exact_setup(const float* f32, float center, float alpha, float p, Geom g, float* gf, float* A,
+                        cudaStream_t s);
+void launch_exact_in(const float* x_user, const float* A, Geom g, float* w, double* acc, cudaStream_t s);
+void launch_exact_mid(const float* S, const float* A, float inv_alpha, Geom g, float* w, double* acc, cudaStream_t s);
+void launch_exact_next(const float* gf, Geom g, float* v, cudaStream_t s);
+void launch_exact_out(const float* S, const float* A, float inv_alpha, Geom g, float* x_user, double* acc,
+                      cudaStream_t s);
 
 // The adjoint's recomputing step with its Q-pass (kernels_fast.cu, mode 6): from the state V_k
 // (internal layout, s = 1/sqrt(*acc_in)) writes the next state to vout exactly as the plain step
@@ -110,6 +113,9 @@ bool launch_adjoint_gpass_fast(const float* vg, float* G, float* Qg, const float
 void launch_apply(const float* x, int x_pitch, float* y, int y_pitch, const float* f32, Geom g,
                   const Taps& tp, float inv_alpha, float p, const double* acc_in, double* acc_out,
                   int* flags, cudaStream_t s, const float* s32 = nullptr);
+
+// x = v over n elements.
+void launch_fill(float* x, int64_t n, float v, cudaStream_t s);
 
 // bf16 copy of a float32 array (n elements).
 void launch_to_bf16(const float* a, __nv_bfloat16* b, int64_t n, cudaStream_t s);

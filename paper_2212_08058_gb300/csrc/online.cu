@@ -22,11 +22,6 @@ struct sfseg_online {
 
 namespace {
 
-__global__ void fill_kernel(float* x, int64_t n, float v) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        x[i] = v;
-}
-
 int check_cuda(cudaError_t e, const char* what) {
     if (e == cudaSuccess) return SFSEG_OK;
     return set_last_error(e == cudaErrorMemoryAllocation ? SFSEG_ERR_OOM : SFSEG_ERR_CUDA,
@@ -89,9 +84,7 @@ int sfseg_online_push(sfseg_online* o, const void* frame, int dtype, const float
                                                 cudaMemcpyDeviceToDevice, s), "window shift"))
             return rc;
     if (o->pushed == 0) {
-        fill_kernel<<<(int)((fr + 255) / 256 < 1024 ? (fr + 255) / 256 : 1024), 256, 0, s>>>(dst + fr * (o->q - 1), fr,
-                                                                                            1.f);
-        count_launches(1);
+        launch_fill(dst + fr * (o->q - 1), fr, 1.f, s);
         if (int rc = check_cuda(cudaGetLastError(), "fill")) return rc;
     } else if (int rc = check_cuda(cudaMemcpyAsync(dst + fr * (o->q - 1), src + fr * (o->q - 1), sizeof(float) * fr,
                                                    cudaMemcpyDeviceToDevice, s), "new frame start")) {

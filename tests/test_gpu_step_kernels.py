@@ -84,3 +84,34 @@ def test_padded_radius_adjoint(sf, T, H, W):
     num = (loss(1e-4) - loss(-1e-4)) / 2e-4
     scale = float(np.abs(np.append(gw, gb)).max())
     assert abs(gw[0] * d[0] + gw[1] * d[1] + gb * d[2] - num) <= 1e-4 * scale
+
+
+def test_exact_operator_in_the_stream_kernel(sf):
+    """The exact (Eq. 1) operator on a volume of the streaming kernel, with the centred series, against
+    the same operator on a crop that the small-volume kernel runs, with the series in f, at voxels
+    whose whole neighbourhood lies in the crop.  Bound: both truncate at 2^-24 of the sum and sum 9 and
+    16 terms of 35 taps each in float32: (9 + 16) * 35 * 2^-24 = 5.2e-5 of max y at most."""
+    T, H, W, r = 6, 343, 561, (1, 3, 3)
+    g = torch.Generator(device="cuda").manual_seed(4)
+    V = torch.rand((1, T, H, W), device="cuda", generator=g)
+    x = torch.rand((T, H, W), device="cuda", generator=g)
+    with sf.PowerIteration(1, T, H, W) as h:
+        h.set_features(V)
+        y = h.apply_exact(x, r)
+    h0, w0, n = 200, 300, 90
+    crop = (slice(None), slice(h0, h0 + n), slice(w0, w0 + n))
+    with sf.PowerIteration(1, T, n, n) as h:
+        h.set_features(V[:, :, h0:h0 + n, w0:w0 + n].contiguous())
+        yc = h.apply_exact(x[crop].contiguous(), r, n_terms=16)
+    a, b = y[crop][:, 3:-3, 3:-3], yc[:, 3:-3, 3:-3]
+    assert float((a - b).abs().max()) <= 5.2e-5 * float(b.abs().max())
+
+
+def test_exact_refusals_stay(sf):
+    """A feature range whose series in f is too long is refused, although the centred one is short."""
+    V = torch.rand((1, 4, 20, 30), device="cuda") * 0.1 + 6.0        # 2 alpha f^2 = 74
+    with sf.PowerIteration(1, 4, 20, 30) as h:
+        h.set_features(V)
+        with pytest.raises(sf.SFSegError) as e:
+            h.apply_exact(torch.rand((4, 20, 30), device="cuda"), (1, 3, 3))
+        assert e.value.status == "UNSUPPORTED"
