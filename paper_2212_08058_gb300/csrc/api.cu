@@ -1047,27 +1047,41 @@ int sfseg_soft_binarize(sfseg_handle* h, const sfseg_neighborhood* nb, int iters
     unsigned* key = reinterpret_cast<unsigned*>(h->scratch + kScrMaxKey);
     const bool fast = fast_step_supported(tp);
     const float* s32 = h->sep ? h->s32 : nullptr;
-    for (int k = 0; k < iters; ++k) {
-        const bool last = k == iters - 1;
-        bool fused = false;   // the stencil took max(y) itself (shared maps, a compiled radius)
-        if (fast && !s32) {
-            SFSEG_CUDA(cudaMemsetAsync(key, 0, sizeof(unsigned), s));
-            if (k == 0) launch_to_state(x_inout, h->f32, nullptr, p, h->g, v, s);
-            fused = launch_iterate_fast_max(v, y, h->f32, h->g, tp, inv_alpha, p, key, h->flags, s);
-            if (!fused && k > 0) return fail(SFSEG_ERR_CUDA, "stencil launch failed");
+    // The steps; x after each of them with every_x, else after the last only.
+    auto steps = [&](bool every_x) -> int {
+        for (int k = 0; k < iters; ++k) {
+            const bool last = k == iters - 1;
+            bool fused = false;   // the stencil took max(y) itself (shared maps, a covered radius)
+            if (fast && !s32) {
+                SFSEG_CUDA(cudaMemsetAsync(key, 0, sizeof(unsigned), s));
+                if (k == 0) launch_to_state(x_inout, h->f32, nullptr, p, h->g, v, s);
+                fused = launch_iterate_fast_max(v, y, h->f32, h->g, tp, inv_alpha, p, key, h->flags, s);
+                if (!fused && k > 0) return fail(SFSEG_ERR_CUDA, "stencil launch failed");
+            }
+            if (!fused) {
+                if (k == 0 || !fast)
+                    launch_apply_user(x_inout, y, v, h->f32, h->g, tp, inv_alpha, p, h->flags, s, s32);
+                else if (!launch_iterate_fast(v, kF32, y, kF32, true, h->f32, h->g, tp, inv_alpha, p, nullptr, nullptr,
+                                              h->flags, s, s32))
+                    return fail(SFSEG_ERR_CUDA, "stencil launch failed");
+                launch_max_key(y, h->N, key, s);
+            }
+            // without a TMA kernel the next step starts from x itself
+            launch_sigmoid_step(y, fused, key, gain, center, h->f32, p, h->g,
+                                last || every_x || !fast ? x_inout : nullptr, (fast && !last) ? v : nullptr,
+                                last ? mask_out : nullptr, h->flags, s, s32);
+            SFSEG_LAUNCHED();
         }
-        if (!fused) {
-            if (k == 0 || !fast)
-                launch_apply_user(x_inout, y, v, h->f32, h->g, tp, inv_alpha, p, h->flags, s, s32);
-            else if (!launch_iterate_fast(v, kF32, y, kF32, true, h->f32, h->g, tp, inv_alpha, p, nullptr, nullptr,
-                                          h->flags, s, s32))
-                return fail(SFSEG_ERR_CUDA, "stencil launch failed");
-            launch_max_key(y, h->N, key, s);
-        }
-        launch_sigmoid_step(y, key, gain, center, h->f32, p, h->g, x_inout, (fast && !last) ? v : nullptr,
-                            last ? mask_out : nullptr, h->flags, s, s32);
-        SFSEG_LAUNCHED();
-    }
+        return SFSEG_OK;
+    };
+    if (int rc = steps(false)) return rc;
+    int fl = 0;
+    SFSEG_CUDA(cudaMemcpyAsync(&fl, h->flags, sizeof(int), cudaMemcpyDeviceToHost, s));
+    SFSEG_CUDA(cudaStreamSynchronize(s));
+    // A step stopped (so did those after it, and x is still the caller's): once more, with x stored by
+    // every step, so that x is left as the step before the stop made it.
+    if ((fl & kFlagTailStop) && fast && iters > 1)
+        if (int rc = steps(true)) return rc;
     return read_flags(h, s);
 }
 

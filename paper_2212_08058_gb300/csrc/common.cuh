@@ -16,6 +16,7 @@ constexpr int kFlagBadFeature = 1;   // a feature value was negative, NaN or Inf
 constexpr int kFlagZeroNorm = 2;     // an iterate norm was exactly zero
 constexpr int kFlagNonfinite = 4;    // an iterate norm was NaN or Inf
 constexpr int kFlagTimeout = 8;      // a bounded wait inside a kernel gave up
+constexpr int kFlagTailStop = 16;    // a soft-binarisation step stopped at its maximum (not an error by itself)
 
 // 1D factors of the separable Gaussian (Sec. 4.2), index d + r for offset d in [-r, r].
 struct Taps {

@@ -205,9 +205,9 @@ __device__ __forceinline__ bool run_of(const Params& P, int s, Run& r) {
 // c_n = (2a)^n / n! and g = f - c for any constant c: with g in f's place and the input v = g^{3j} w,
 // its three filtered signals are the series terms n = 3j (G*v), 3j + 1 (G*(g v)) and 3j + 2
 // (G*(g^2 v)); it adds t = s g^{3j} (c_{3j} G*v + g (c_{3j+1} G*(g v) + g c_{3j+2} G*(g^2 v))) to out
-// (writes it when j = 0).  All in the internal layout.  MODE 8 is the step (MODE 0) that also takes the
-// largest of its outputs and adds it to P.maxkey (atomicMax of the order key, one per CTA): the
-// maximum a soft-binarisation step (Alg. 1 step 3) scales by, without a pass of its own.
+// (writes it when j = 0).  All in the internal layout.  MODE 8 writes x~ in the
+// internal layout and adds the largest of its outputs to P.maxkey (atomicMax of the order key, one per
+// warp): the maximum a soft-binarisation step (Alg. 1 step 3) scales by, without a pass of its own.
 template <int RT, int RH, int RW, typename TS, typename TVO, bool OUT_X, bool SEP, int MODE>
 __global__ void __launch_bounds__(NTHR, 1)
 iter_stream(const __grid_constant__ Maps M, const __grid_constant__ Params P) {
@@ -524,7 +524,7 @@ iter_stream(const __grid_constant__ Maps M, const __grid_constant__ Params P) {
                             const float2 xt = mul2(mul2(s2, u), B);
                             part = fma2(xt, xt, part);
                             if constexpr (MODE == 8) tmax = fmaxf(tmax, fmaxf(xt.x, xt.y));
-                            outv[m] = OUT_X ? xt : mul2(u, xt);
+                            outv[m] = (OUT_X || MODE == 8) ? xt : mul2(u, xt);
                             if constexpr (MODE == 4) outq[m] = xt;
                             if constexpr (MODE == 6) {
                                 const float2 a1 = fma2(f2(P.p), ee, mul2(f2(-2.f), mul2(fv, fv)));

@@ -312,7 +312,7 @@ iter_tile(const __grid_constant__ CUtensorMap mv, const __grid_constant__ CUtens
                     const float2 xt = mul2(mul2(s2, u), B);
                     part = fma2(xt, xt, part);
                     if constexpr (MODE == 8) tmax = fmaxf(tmax, fmaxf(xt.x, xt.y));
-                    outv[m] = OUT_X ? xt : mul2(u, xt);
+                    outv[m] = (OUT_X || MODE == 8) ? xt : mul2(u, xt);
                     if constexpr (MODE == 4) outq[m] = xt;
                     if constexpr (MODE == 6) {
                         const float2 a1 = fma2(f2(P.p), e, mul2(f2(-2.f), mul2(fv, fv)));

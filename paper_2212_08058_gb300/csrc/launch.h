@@ -46,7 +46,7 @@ bool launch_iterate_fast(const void* vin, int vin_type, void* out, int out_type,
                          const Geom& g, const Taps& tp, float inv_alpha, float p, const double* acc_in,
                          double* acc_out, int* flags, cudaStream_t s, const float* s32 = nullptr);
 
-// The TMA step from the state vin (internal layout, float32) to y = A x in the caller layout that
+// The TMA step from the state vin (internal layout, float32) to y = A x in the internal layout that
 // also adds the order key of its largest output to *maxkey (atomicMax; zero it first): a
 // soft-binarisation step's maximum without a pass of its own.  No norm scaling.  False (nothing
 // launched) for a radius without a compiled kernel.
@@ -134,10 +134,12 @@ void launch_upsample(const float* xc, int Tc, int Hc, int Wc, int pt, int ph, in
 void launch_scale_by_max(float* x, int64_t n, unsigned* key, cudaStream_t s);
 
 // Soft-binarisation step pieces (kernels_tail.cu): *key = order-preserving key of max(y) over
-// n caller-layout values (the key is reset first); x = sigmoid(gain (y / max y - center)) with
-// optional v = u * x (internal layout) and mask = (x > 1/2).
+// n caller-layout values (the key is reset first); x = sigmoid(gain (y / max y - center)), y in the
+// internal layout or the caller's, with any of v = u * x (internal layout), x and mask = (x > 1/2)
+// (caller layout, nullable).  A maximum that is not positive and finite sets its flag and
+// kFlagTailStop and leaves the outputs alone.
 void launch_max_key(const float* y, int64_t n, unsigned* key, cudaStream_t s);
-void launch_sigmoid_step(const float* y, const unsigned* key, float gain, float center, const float* f32, float p,
+void launch_sigmoid_step(const float* y, bool y_internal, const unsigned* key, float gain, float center, const float* f32, float p,
                          Geom g, float* x, float* v, unsigned char* mask, int* flags, cudaStream_t s,
                          const float* s32 = nullptr);
 

@@ -64,7 +64,7 @@ bool step_dispatch(const StepArgs& a) {
         case kGPass: return K::template launch<float, float, false, false, kGPass>(a);
         case kStepQ: return K::template launch<float, float, false, false, kStepQ>(a);
         case kExactTerm: return K::template launch<float, float, false, false, kExactTerm>(a);
-        case kStepMax: return K::template launch<float, float, true, false, kStepMax>(a);
+        case kStepMax: return K::template launch<float, float, false, false, kStepMax>(a);
     }
     return false;
 }
