@@ -222,7 +222,7 @@ __global__ void __launch_bounds__(ConvCfg<CIN, COUT, FR>::NTHR, 1)
 conv3d_tc(const __grid_constant__ CUtensorMap xin, ConvArgs a) {
     using C = ConvCfg<CIN, COUT, FR>;
     extern __shared__ __align__(128) unsigned char sm_raw[];
-    unsigned char* sm = (unsigned char*)(((uintptr_t)sm_raw + 127) & ~(uintptr_t)127);
+    unsigned char* sm = sm_raw + (-su32(sm_raw) & 127u);   // an offset keeps the shared address space
     unsigned char* wsm = sm;                                   // weights
     unsigned char* ring = sm + C::WBYTES;                      // the input-row slots
     uint64_t* bar = reinterpret_cast<uint64_t*>(ring + C::NS * C::SLOT_BYTES);
@@ -496,7 +496,7 @@ __global__ void __launch_bounds__(LastCfg<FR>::NTHR, LastCfg<FR>::CTAS)
 conv_last_tc(const __grid_constant__ CUtensorMap xin, LastArgs a) {
     using L = LastCfg<FR>;
     extern __shared__ __align__(128) unsigned char sm_raw[];
-    unsigned char* sm = (unsigned char*)(((uintptr_t)sm_raw + 127) & ~(uintptr_t)127);
+    unsigned char* sm = sm_raw + (-su32(sm_raw) & 127u);   // an offset keeps the shared address space
     unsigned char* wsm = sm;
     unsigned char* ring = sm + LT_BBYTES;
     unsigned char* xs0 = ring + L::NS * L::SLOT;            // [FR][XS1]
@@ -724,7 +724,7 @@ __global__ void __launch_bounds__(NTHR, 1)
 wgrad_tc(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUtensorMap dzmap, WgArgs a) {
     using C = WgCfg<NCI, NCO>;
     extern __shared__ __align__(128) unsigned char sm_raw[];
-    unsigned char* sm = (unsigned char*)(((uintptr_t)sm_raw + 127) & ~(uintptr_t)127);
+    unsigned char* sm = sm_raw + (-su32(sm_raw) & 127u);   // an offset keeps the shared address space
     uint64_t* bar = reinterpret_cast<uint64_t*>(sm + WG_NS * C::STAGE);
     uint64_t* full = bar;               // [WG_NS]
     uint64_t* empty = bar + WG_NS;      // [WG_NS]
@@ -855,12 +855,29 @@ wgrad_tc(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUten
 
 // Sum of the CTAs' partial sums in a fixed order: dW[co][tap][ci] with tap = 9 (dt + 1) +
 // 3 (dh + 1) + (dw + 1) from row block j = dh + 1, dz frame s = 1 - dt; db[co] from the constant
-// row block (m = 96) of the dz frame s = 1 (the others repeat it).
+// row block (m = 96) of the dz frame s = 1 (the others repeat it).  A block sums 32 values, each of its
+// warps every kRedWarps-th partial: one thread per value walked 152 partials 147 KB apart, 28 us of
+// memory latency for 22 MB.  Sums are kept as hi + lo, the error-free transformation of each addition
+// (Knuth's TwoSum), to about 48 bits like FP64 would, at FP32 rate.
+constexpr int kRedWarps = 8;
+struct TwoFloat {
+    float hi = 0.f, lo = 0.f;
+    __device__ __forceinline__ void add(float v) {
+        const float t = __fadd_rn(hi, v), z = __fsub_rn(t, hi);
+        lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(t, z)), __fsub_rn(v, z)));
+        hi = t;
+    }
+};
 template <int NCI, int NCO>
-__global__ void wgrad_reduce(const float* part, int nparts, int cout, int cin, float* dW, float* db) {
+__global__ void __launch_bounds__(32 * kRedWarps)
+wgrad_reduce(const float* part, int nparts, int cout, int cin, float* dW, float* db) {
     using C = WgCfg<NCI, NCO>;
+    __shared__ TwoFloat sums[kRedWarps][32];
     const int total = cout * 27 * cin;
-    for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < total + cout; idx += gridDim.x * blockDim.x) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int idx = blockIdx.x * 32 + lane;
+    TwoFloat acc;
+    if (idx < total + cout) {
         int n, m, dw;
         if (idx < total) {
             const int ci = idx % cin, tap = (idx / cin) % 27, co = idx / (cin * 27);
@@ -874,19 +891,19 @@ __global__ void wgrad_reduce(const float* part, int nparts, int cout, int cin, f
             n = NCO * 8 + co;
             m = 96;
         }
-        // hi + lo: the error-free transformation of each addition (Knuth's TwoSum), which keeps the
-        // sum to about 48 bits like FP64 would, at FP32 rate
-        float hi = 0.f, lo = 0.f;
-#pragma unroll 8
-        for (int p = 0; p < nparts; ++p) {
-            const float v = part[(size_t)p * C::PART + ((size_t)dw * C::N + n) * 128 + m];
-            const float t = __fadd_rn(hi, v), z = __fsub_rn(t, hi);
-            lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(t, z)), __fsub_rn(v, z)));
-            hi = t;
+        const float* p0 = part + ((size_t)dw * C::N + n) * 128 + m;
+#pragma unroll 4
+        for (int p = warp; p < nparts; p += kRedWarps) acc.add(p0[(size_t)p * C::PART]);
+    }
+    sums[warp][lane] = acc;
+    __syncthreads();
+    if (warp == 0 && idx < total + cout) {
+        for (int w = 1; w < kRedWarps; ++w) {
+            acc.add(sums[w][lane].hi);
+            acc.lo = __fadd_rn(acc.lo, sums[w][lane].lo);
         }
-        const float acc = hi + lo;
-        if (idx < total) dW[idx] = acc;
-        else db[idx - total] = acc;
+        if (idx < total) dW[idx] = acc.hi + acc.lo;
+        else db[idx - total] = acc.hi + acc.lo;
     }
 }
 
@@ -1326,7 +1343,8 @@ int run_wgrad(sfseg_net* n, int cout, int cin, const __nv_bfloat16* dz, const __
     a.per = (a.units + num_sms() - 1) / num_sms();
     const int grid = (a.units + a.per - 1) / a.per;   // every CTA gets at least one unit
     k<<<grid, NTHR, Cf::SMEM, s>>>(xm, dm, a);
-    wgrad_reduce<NCI, NCO><<<(cout * 27 * cin + cout + 255) / 256, 256, 0, s>>>(n->wg_part, grid, cout, cin, dW, db);
+    wgrad_reduce<NCI, NCO><<<(cout * 27 * cin + cout + 31) / 32, 32 * kRedWarps, 0, s>>>(n->wg_part, grid, cout, cin,
+                                                                                        dW, db);
     count_launches(2);
     NET_CUDA(cudaGetLastError());
     return SFSEG_OK;
