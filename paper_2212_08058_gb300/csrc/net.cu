@@ -12,9 +12,12 @@
 //   K = 16 input channels per instruction.  Each input row is read once: its 9 (dt, dw) taps x
 //   C_in/16 MMAs each carry the three taps along h at once (N = 3 x output channels, D over the
 //   accumulators of the three output rows it feeds, a ring of blocks in TMEM).
-// The A operand is read straight from a TMA-filled ring of input rows in the canonical
-// no-swizzle K-major layout ([8-channel chunk][frames][130 voxels][8 channels]); a tap's shift
-// along w is a 16-byte offset of the descriptor's start address, along t a 2080-byte offset.
+// The A operand is read straight from a TMA-filled ring of input rows, [frames][130 voxels][channels]
+// in the K-major layout whose swizzle is as wide as a voxel (64 bytes at 32 channels, 32 at 16): one
+// copy per row, a whole voxel per request.  A tap's shift along w is one voxel's offset of the
+// descriptor's start address, along t a frame's.  (With one 16-byte-wide copy per 8 channels in the
+// no-swizzle layout every 32-byte sector was fetched twice: 24x1080x1920 8246 us for the network, 7505
+// now.)
 // All weights of the layer stay in shared memory.  A CTA computes up to three consecutive output
 // frames from input slots of two more frames: one warp issues the TMA copies, one per output
 // frame issues its MMAs (each into its part of TMEM), four per frame read each finished row's
@@ -98,6 +101,13 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t by
 __device__ __forceinline__ uint64_t sdesc(uint32_t saddr, uint32_t lbo, uint32_t sbo) {
     return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)((lbo >> 4) & 0x3FFFu) << 16) |
            ((uint64_t)((sbo >> 4) & 0x3FFFu) << 32) | (1ull << 46);
+}
+// Shared-memory matrix descriptor: K-major rows of `row` = 64 or 32 bytes, packed, with the swizzle of
+// that width (the 16-byte pieces of a row XORed with address bits 7.. on, as a TMA copy with the same
+// swizzle writes them: by address, so a start address may be any row).
+__device__ __forceinline__ uint64_t sdesc_rows(uint32_t saddr, uint32_t row) {
+    return (uint64_t)((saddr & 0x3FFFFu) >> 4) | (1ull << 16) | ((uint64_t)(8 * row >> 4) << 32) | (1ull << 46) |
+           ((row == 64 ? 4ull : 6ull) << 61);
 }
 // Instruction descriptor, kind::f16: bf16 A and B (K-major), fp32 D, M = 128, N = n.
 __host__ __device__ constexpr uint32_t idesc_bf16(int n) {
@@ -195,11 +205,11 @@ template <int CIN, int COUT, int FR_>
 struct ConvCfg {
     static constexpr int FR = FR_;                            // output frames per CTA
     static constexpr int NF = FR + 2;                         // frames per input slot
-    static constexpr int NCH = CIN / 8;                       // 8-channel chunks of A
     static constexpr int KS = CIN / 16;                       // MMAs per tap
-    static constexpr int CHUNK_DATA = NF * RW * 16;           // one 8-channel chunk of NF frames
-    static constexpr int CHUNK = (CHUNK_DATA + 127) / 128 * 128;   // its stride (128-byte aligned TMA target)
-    static constexpr int SLOT_BYTES = NCH * CHUNK;
+    static constexpr int VB = CIN * 2;                        // bytes of a voxel: one row of A
+    static constexpr int FB = RW * VB;                        // one frame of an input row
+    static constexpr int SLOT_DATA = NF * FB;
+    static constexpr int SLOT_BYTES = (SLOT_DATA + 511) / 512 * 512;   // the swizzle repeats every 512 bytes
     static constexpr int WBYTES = 27 * KS * 2 * COUT * 16;    // packed weights
     static constexpr int RING = (512 / FR) / 32 * 32;         // TMEM columns of one output frame
     static constexpr int R = RING / COUT;                     // accumulator blocks in its ring
@@ -209,7 +219,7 @@ struct ConvCfg {
     static constexpr int NTHR = 32 * (1 + FR + 4 * FR);       // producer, issuers, 4 epilogue warps per frame
     // full[NS], empty[NS], accf[FR][R], acce[FR][R], wbar, drain[FR]
     static constexpr int NB = 2 * NS + 2 * FR * R + 1 + FR;
-    static constexpr int SMEM_NEED = WBYTES + NS * SLOT_BYTES + NB * 8 + 16 + 128;
+    static constexpr int SMEM_NEED = WBYTES + NS * SLOT_BYTES + NB * 8 + 16 + 512;
     // at least 120 KB so that one CTA holds the SM's tensor memory alone
     static constexpr int SMEM = SMEM_NEED > 120 * 1024 ? SMEM_NEED : 120 * 1024;
     static_assert(FR >= 1 && FR <= 3, "one to three output frames per CTA");
@@ -222,7 +232,7 @@ __global__ void __launch_bounds__(ConvCfg<CIN, COUT, FR>::NTHR, 1)
 conv3d_tc(const __grid_constant__ CUtensorMap xin, ConvArgs a) {
     using C = ConvCfg<CIN, COUT, FR>;
     extern __shared__ __align__(128) unsigned char sm_raw[];
-    unsigned char* sm = sm_raw + (-su32(sm_raw) & 127u);   // an offset keeps the shared address space
+    unsigned char* sm = sm_raw + (-su32(sm_raw) & 511u);   // an offset keeps the shared address space
     unsigned char* wsm = sm;                                   // weights
     unsigned char* ring = sm + C::WBYTES;                      // the input-row slots
     uint64_t* bar = reinterpret_cast<uint64_t*>(ring + C::NS * C::SLOT_BYTES);
@@ -291,9 +301,8 @@ conv3d_tc(const __grid_constant__ CUtensorMap xin, ConvArgs a) {
                 const int s = i % C::NS;
                 if (i >= C::NS && !mb_wait(&empty[s], (uint32_t)((i / C::NS - 1) & 1), a.flags)) break;
                 issued = i + 1;
-                mb_expect(&full[s], C::NCH * C::CHUNK_DATA);
-                unsigned char* dst = ring + s * C::SLOT_BYTES;
-                for (int k = 0; k < C::NCH; ++k) tma4(dst + k * C::CHUNK, &xin, &full[s], 8 * k, w0 - 1, hs - 1 + i, t0 - 1);
+                mb_expect(&full[s], C::SLOT_DATA);
+                tma4(ring + s * C::SLOT_BYTES, &xin, &full[s], 0, w0 - 1, hs - 1 + i, t0 - 1);
             }
         }
     } else if (epi < 0) {
@@ -319,7 +328,7 @@ conv3d_tc(const __grid_constant__ CUtensorMap xin, ConvArgs a) {
                 const int n1 = min(nrow, C::R - b0), n2 = nrow - n1;   // before and after the wrap
                 const uint32_t id1 = idesc_bf16(n1 * COUT), id2 = idesc_bf16((n2 > 0 ? n2 : 1) * COUT);
                 const uint32_t d1 = dbase + (uint32_t)(b0 * COUT), d2 = dbase;
-                const uint64_t a0 = sdesc(rbase + (uint32_t)((i % C::NS) * C::SLOT_BYTES + q * RW * 16), C::CHUNK, 128);
+                const uint64_t a0 = sdesc_rows(rbase + (uint32_t)((i % C::NS) * C::SLOT_BYTES + q * C::FB), C::VB);
                 // B of rows dh0 .. and of the rows after the wrap: same tiles, later start rows
                 const uint64_t bA = sdesc(wbase + (uint32_t)(dh0 * COUT * 16), 3 * COUT * 16, 128);
                 const uint64_t bB = sdesc(wbase + (uint32_t)((dh0 + n1) * COUT * 16), 3 * COUT * 16, 128);
@@ -332,7 +341,7 @@ conv3d_tc(const __grid_constant__ CUtensorMap xin, ConvArgs a) {
                     for (int dw = 0; dw < 3; ++dw)
 #pragma unroll
                         for (int ks = 0; ks < C::KS; ++ks) {
-                            const uint64_t ad = a0 + (uint64_t)((2 * ks * C::CHUNK + dt * RW * 16 + dw * 16) >> 4);
+                            const uint64_t ad = a0 + (uint64_t)((dt * C::FB + dw * C::VB + ks * 32) >> 4);
                             const uint64_t toff = (uint64_t)((((dt * 3 + dw) * C::KS + ks) * TILE) >> 4);
                             umma(d1, ad, bA + toff, id1, 1u);
                         }
@@ -343,7 +352,7 @@ conv3d_tc(const __grid_constant__ CUtensorMap xin, ConvArgs a) {
                         for (int dw = 0; dw < 3; ++dw)
 #pragma unroll
                             for (int ks = 0; ks < C::KS; ++ks) {
-                                const uint64_t ad = a0 + (uint64_t)((2 * ks * C::CHUNK + dt * RW * 16 + dw * 16) >> 4);
+                                const uint64_t ad = a0 + (uint64_t)((dt * C::FB + dw * C::VB + ks * 32) >> 4);
                                 const uint64_t toff = (uint64_t)((((dt * 3 + dw) * C::KS + ks) * TILE) >> 4);
                                 umma(d2, ad, bB + toff, id2, 1u);
                             }
@@ -473,9 +482,9 @@ struct LastArgs {
 template <int FR>
 struct LastCfg {
     static constexpr int NF = FR + 2;                     // frames per input slot
-    static constexpr int CHUNK_DATA = NF * RW * 16;       // one 8-channel chunk of NF frames
-    static constexpr int CHUNK = (CHUNK_DATA + 127) / 128 * 128;
-    static constexpr int SLOT = 4 * CHUNK;                // one input row: 4 chunks of 8 channels
+    static constexpr int FB = RW * 64;                    // one frame of an input row: 32 channels a voxel
+    static constexpr int SLOT_DATA = NF * FB;
+    static constexpr int SLOT = (SLOT_DATA + 511) / 512 * 512;
     static constexpr int CTAS = FR == 1 ? 2 : 1;          // CTAs per SM
     static constexpr int COLS = 512 / CTAS;               // TMEM columns of the CTA
     static constexpr int R = COLS / (16 * FR);            // rows in the ring (FR blocks each)
@@ -485,7 +494,7 @@ struct LastCfg {
     static constexpr int XS1 = 2 * 3 * 128 * 4 + 2 * 4 * 4;
     static constexpr int XS = FR * XS1;
     static constexpr int NB = 2 * NS + 2 * FR * R + 2;    // full, empty, accf[FR][R], acce[FR][R], wbar, drain
-    static constexpr int SMEM = LT_BBYTES + NS * SLOT + XS + NB * 8 + 16 + 128;
+    static constexpr int SMEM = LT_BBYTES + NS * SLOT + XS + NB * 8 + 16 + 512;
     static_assert(R >= 4, "accumulator ring");
     static_assert(FR <= 4, "named barriers 1..FR");
     static_assert(SMEM * CTAS <= 227 * 1024, "shared memory");
@@ -496,7 +505,7 @@ __global__ void __launch_bounds__(LastCfg<FR>::NTHR, LastCfg<FR>::CTAS)
 conv_last_tc(const __grid_constant__ CUtensorMap xin, LastArgs a) {
     using L = LastCfg<FR>;
     extern __shared__ __align__(128) unsigned char sm_raw[];
-    unsigned char* sm = sm_raw + (-su32(sm_raw) & 127u);   // an offset keeps the shared address space
+    unsigned char* sm = sm_raw + (-su32(sm_raw) & 511u);   // an offset keeps the shared address space
     unsigned char* wsm = sm;
     unsigned char* ring = sm + LT_BBYTES;
     unsigned char* xs0 = ring + L::NS * L::SLOT;            // [FR][XS1]
@@ -554,9 +563,8 @@ conv_last_tc(const __grid_constant__ CUtensorMap xin, LastArgs a) {
                 const int s = i % L::NS;
                 if (i >= L::NS && !mb_wait(&empty[s], (uint32_t)((i / L::NS - 1) & 1), a.flags)) break;
                 issued = i + 1;
-                mb_expect(&full[s], 4 * L::CHUNK_DATA);
-                unsigned char* dst = ring + s * L::SLOT;
-                for (int k = 0; k < 4; ++k) tma4(dst + k * L::CHUNK, &xin, &full[s], 8 * k, w0 - 1, hs - 1 + i, t0 - 1);
+                mb_expect(&full[s], L::SLOT_DATA);
+                tma4(ring + s * L::SLOT, &xin, &full[s], 0, w0 - 1, hs - 1 + i, t0 - 1);
             }
         }
     } else if (warp == 1) {
@@ -572,14 +580,14 @@ conv_last_tc(const __grid_constant__ CUtensorMap xin, LastArgs a) {
                         ok = mb_wait(&acce[q * L::R + i % L::R], (uint32_t)(((i - L::R) / L::R) & 1), a.flags);
                 if (!ok) break;
                 tc_fence_after();
-                const uint64_t a0 = sdesc(rbase + (uint32_t)((i % L::NS) * L::SLOT), L::CHUNK, 128);
+                const uint64_t a0 = sdesc_rows(rbase + (uint32_t)((i % L::NS) * L::SLOT), 64);
                 // row i's blocks of all FR output frames (those past the last frame are not read)
                 const uint32_t d = tmem + (uint32_t)((i % L::R) * FR * 16);
 #pragma unroll
                 for (int sf = 0; sf < L::NF; ++sf)   // slot frame t0 - 1 + sf
 #pragma unroll
                     for (int ks = 0; ks < 2; ++ks) {
-                        const uint64_t ad = a0 + (uint64_t)((2 * ks * L::CHUNK + sf * RW * 16) >> 4);
+                        const uint64_t ad = a0 + (uint64_t)((sf * L::FB + ks * 32) >> 4);
                         const uint64_t bd = sdesc(wbase + (uint32_t)(2 * ks * LT_CH + (5 - sf) * 256), LT_CH, 128);
                         umma(d, ad, bd, ID, (sf | ks) ? 1u : 0u);
                     }
@@ -1059,18 +1067,18 @@ EncodeFn encode() {
     return fn;
 }
 
-// 4D map over a channels-last bf16 activation [T][H][W][C]; box = 8 channels x 130 voxels x
-// 1 row x 3 frames (one A chunk of one input row).
-bool act_map(CUtensorMap* m, const void* base, int C, int T, int H, int W, int frames = 3) {
+// 4D map over a channels-last bf16 activation [T][H][W][C], C = 16 or 32; box = all channels x 130
+// voxels x 1 row x `frames`, each voxel's 32 or 64 bytes swizzled (the A operand's rows).
+bool act_map(CUtensorMap* m, const void* base, int C, int T, int H, int W, int frames) {
     EncodeFn fn = encode();
     if (!fn) return false;
     cuuint64_t dims[4] = {(cuuint64_t)C, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)T};
     cuuint64_t str[3] = {(cuuint64_t)C * 2, (cuuint64_t)C * 2 * W, (cuuint64_t)C * 2 * W * H};
-    cuuint32_t box[4] = {8, (cuuint32_t)RW, 1, (cuuint32_t)frames};
+    cuuint32_t box[4] = {(cuuint32_t)C, (cuuint32_t)RW, 1, (cuuint32_t)frames};
     cuuint32_t es[4] = {1, 1, 1, 1};
     return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, str, box, es,
-              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+              CU_TENSOR_MAP_INTERLEAVE_NONE, C == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B,
+              CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 // 4D map over a channels-last bf16 activation [T][H][W][C] with a box of 8 channels x bw voxels
