@@ -686,21 +686,17 @@ __global__ void pack_last_taps(const float* W, __nv_bfloat16* out) {
 // along w).  With the x frame fixed, the taps (dt, dh, dw) of one unit form three products, one
 // per dw:
 //   D_dw[(j, ci), (s, co)] += sum_k x[t, h - 1 + j, w0 + k + dw - 1, ci] * dz[t - 1 + s, h, w0 + k, co]
-// for j = dh + 1 in 0..2 and s = 1 - dt in 0..2: M = 128 stacks four 32-channel row blocks of x
-// (the fourth is a constant 1, so its rows of D sum dz: the bias gradient), N stacks the three dz
-// frames (3 x 32 channels; 3 x 16 for the last layer's one channel padded to 16).  Both operands
-// are read in the MN-major layout straight from the TMA copies of the channels-last activations:
-// [block][8-channel chunk][voxels][8 channels], where a core matrix is 8 voxels (K) x 8 channels
-// (16 bytes) and a shift by one voxel along w is a 16-byte offset of the descriptor's start.  In
-// the descriptor of this no-swizzle MN-major layout the leading-dimension offset is the step
-// between groups of 8 voxels along K (128 bytes) and the stride-dimension offset the step between
-// 8-channel chunks along M or N (measured: the other assignment gives wrong sums).
+// for j = dh + 1 in 0..2 and s = 1 - dt in 0..2: M = 128 stacks the three row blocks of x (32 or 16
+// channels each) and fills up with blocks of a constant 1, whose rows of D sum dz: the bias gradient;
+// N stacks the three dz frames (3 x 32 channels; 3 x 16 for the last layer's one channel padded to
+// 16).  Both operands are read in the MN-major layout straight from TMA copies of the channels-last
+// activations, [block][voxels][channels] with the swizzle as wide as a voxel (64 or 32 bytes): in the
+// descriptor the leading-dimension offset is the step between blocks along M or N and the
+// stride-dimension offset the step between groups of 8 voxels along K; a shift by one voxel along w is
+// one voxel's offset of the start address.  A unit takes two copies, three x rows and three dz frames.
 // Every unit of a CTA accumulates into the same TMEM columns; at the end the CTA writes its
 // partial sums to a scratch slice and a second kernel adds the slices in a fixed order.
 constexpr int WG_XV = MT + 2;                              // x voxels per row (w halo 1)
-constexpr int WG_CHA = (WG_XV * 16 + 127) / 128 * 128;     // A chunk stride (2176 B)
-constexpr int WG_CHB = MT * 16;                            // B chunk stride (2048 B)
-constexpr int WG_A_BYTES = 16 * WG_CHA;                    // 4 row blocks x 4 chunks
 #ifndef SFSEG_NET_WG_NS
 #define SFSEG_NET_WG_NS 3
 #endif
@@ -709,12 +705,18 @@ constexpr int WG_NS = SFSEG_NET_WG_NS;   // stages (2 measured 4 % slower; 4 exc
 template <int NCI, int NCO>
 struct WgCfg {
     static constexpr int N = 3 * NCO * 8;                  // 96 or 48
-    static constexpr int B_BYTES = 3 * NCO * WG_CHB;
-    static constexpr int STAGE = WG_A_BYTES + B_BYTES;
+    static constexpr int XC = NCI * 8;                     // channels of a row block of A
+    static constexpr int XB = XC * 2, ZB = NCO * 16;       // bytes of an x voxel, of a dz voxel
+    static constexpr int ABLK = WG_XV * XB;                // a row block of A
+    static constexpr int BBLK = MT * ZB;                   // a dz frame of B
+    static constexpr int A_BYTES = 128 / XC * ABLK;        // three row blocks, then ones
+    static constexpr int B_BYTES = 3 * BBLK;
+    static constexpr int STAGE = (A_BYTES + B_BYTES + 511) / 512 * 512;
+    static_assert(A_BYTES % 512 == 0, "B starts where the swizzle does");
     static constexpr int TMEM_COLS = 3 * N <= 256 ? 256 : 512;
     // (the barriers sit after the stages; 8 KB more keep every descriptor offset inside the
     // allocation whatever the operand reach)
-    static constexpr int SMEM = WG_NS * STAGE + (2 * WG_NS + 2) * 8 + 16 + 128 + 8192;
+    static constexpr int SMEM = WG_NS * STAGE + (2 * WG_NS + 2) * 8 + 16 + 512 + 8192;
     static constexpr int PART = 3 * N * 128;               // floats of one CTA's partial sums
 };
 
@@ -724,6 +726,12 @@ struct WgArgs {
     int* flags;
 };
 
+// Shared-memory matrix descriptor: MN-major, voxels of `row` = 64 or 32 bytes with the swizzle of that
+// width, `block` bytes between blocks of that many channels along M or N.
+__device__ __forceinline__ uint64_t sdesc_mn(uint32_t saddr, uint32_t row, uint32_t block) {
+    return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)(block >> 4) << 16) | ((uint64_t)(8 * row >> 4) << 32) |
+           (1ull << 46) | ((row == 64 ? 4ull : 6ull) << 61);
+}
 // Instruction descriptor, kind::f16: bf16 A and B, both MN-major, fp32 D, M = 128, N = n.
 __host__ __device__ constexpr uint32_t idesc_bf16_mn(int n) { return idesc_bf16(n) | (1u << 15) | (1u << 16); }
 
@@ -732,7 +740,7 @@ __global__ void __launch_bounds__(NTHR, 1)
 wgrad_tc(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUtensorMap dzmap, WgArgs a) {
     using C = WgCfg<NCI, NCO>;
     extern __shared__ __align__(128) unsigned char sm_raw[];
-    unsigned char* sm = sm_raw + (-su32(sm_raw) & 127u);   // an offset keeps the shared address space
+    unsigned char* sm = sm_raw + (-su32(sm_raw) & 511u);   // an offset keeps the shared address space
     uint64_t* bar = reinterpret_cast<uint64_t*>(sm + WG_NS * C::STAGE);
     uint64_t* full = bar;               // [WG_NS]
     uint64_t* empty = bar + WG_NS;      // [WG_NS]
@@ -745,15 +753,11 @@ wgrad_tc(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUten
     const int u0 = blockIdx.x * a.per, u1 = min(a.units, u0 + a.per);
     const int nu = max(u1 - u0, 0);
 
-    // the constant row block (ones) of every stage, and the channel chunks an input with fewer
-    // than 32 channels (NCI < 4) does not fill (zeros); no copy ever writes either
-    for (int i = threadIdx.x; i < WG_NS * 16 * WG_CHA / 16; i += blockDim.x) {
-        const int st = i / (16 * WG_CHA / 16), r = i % (16 * WG_CHA / 16);
-        const int blk = r / (WG_CHA / 16);          // (j, c) block: j = blk / 4, c = blk % 4
-        uint4* p = reinterpret_cast<uint4*>(sm + st * C::STAGE) + r;
-        if (blk >= 12) *p = make_uint4(0x3F803F80u, 0x3F803F80u, 0x3F803F80u, 0x3F803F80u);   // bf16 1.0 x 8
-        else if (blk % 4 >= NCI) *p = make_uint4(0u, 0u, 0u, 0u);
-    }
+    // the constant row blocks (ones) of every stage; no copy ever writes them
+    constexpr int kOnes = (C::A_BYTES - 3 * C::ABLK) / 16;
+    for (int i = threadIdx.x; i < WG_NS * kOnes; i += blockDim.x)
+        reinterpret_cast<uint4*>(sm + i / kOnes * C::STAGE + 3 * C::ABLK)[i % kOnes] =
+            make_uint4(0x3F803F80u, 0x3F803F80u, 0x3F803F80u, 0x3F803F80u);   // bf16 1.0 x 8
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     if (threadIdx.x == 0) {
         for (int i = 0; i < WG_NS; ++i) {
@@ -789,13 +793,9 @@ wgrad_tc(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUten
                 const int h = u % a.H, t = u / a.H;
                 const int w0 = ws * MT;
                 unsigned char* st = sm + s * C::STAGE;
-                mb_expect(&full[s], 3u * NCI * (uint32_t)(WG_XV * 16) + 3u * NCO * (uint32_t)WG_CHB);
-                for (int j = 0; j < 3; ++j)
-                    for (int c = 0; c < NCI; ++c)
-                        tma4(st + (j * 4 + c) * WG_CHA, &xmap, &full[s], 8 * c, w0 - 1, h - 1 + j, t);
-                for (int f = 0; f < 3; ++f)
-                    for (int c = 0; c < NCO; ++c)
-                        tma4(st + WG_A_BYTES + (f * NCO + c) * WG_CHB, &dzmap, &full[s], 8 * c, w0, h, t - 1 + f);
+                mb_expect(&full[s], 3u * C::ABLK + 3u * C::BBLK);
+                tma4(st, &xmap, &full[s], 0, w0 - 1, h - 1, t);
+                tma4(st + C::A_BYTES, &dzmap, &full[s], 0, w0, h, t - 1);
             }
         }
     } else if (warp == 1) {
@@ -809,13 +809,13 @@ wgrad_tc(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUten
                     break;
                 }
                 tc_fence_after();
-                const uint32_t sa = base + (uint32_t)(s * C::STAGE), sb = sa + WG_A_BYTES;
+                const uint32_t sa = base + (uint32_t)(s * C::STAGE), sb = sa + C::A_BYTES;
 #pragma unroll
                 for (int dw = 0; dw < 3; ++dw)
 #pragma unroll
                     for (int kk = 0; kk < MT / 16; ++kk) {
-                        const uint64_t ad = sdesc(sa + (uint32_t)((kk * 16 + dw) * 16), 128, WG_CHA);
-                        const uint64_t bd = sdesc(sb + (uint32_t)(kk * 16 * 16), 128, WG_CHB);
+                        const uint64_t ad = sdesc_mn(sa + (uint32_t)((kk * 16 + dw) * C::XB), C::XB, C::ABLK);
+                        const uint64_t bd = sdesc_mn(sb + (uint32_t)(kk * 16 * C::ZB), C::ZB, C::BBLK);
                         umma(tmem + (uint32_t)(dw * C::N), ad, bd, ID, (i > 0 || kk > 0) ? 1u : 0u);
                     }
                 umma_commit(&empty[s]);
@@ -862,8 +862,8 @@ wgrad_tc(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUten
 }
 
 // Sum of the CTAs' partial sums in a fixed order: dW[co][tap][ci] with tap = 9 (dt + 1) +
-// 3 (dh + 1) + (dw + 1) from row block j = dh + 1, dz frame s = 1 - dt; db[co] from the constant
-// row block (m = 96) of the dz frame s = 1 (the others repeat it).  A block sums 32 values, each of its
+// 3 (dh + 1) + (dw + 1) from row block j = dh + 1, dz frame s = 1 - dt; db[co] from the first constant
+// row block of the dz frame s = 1 (the others repeat it).  A block sums 32 values, each of its
 // warps every kRedWarps-th partial: one thread per value walked 152 partials 147 KB apart, 28 us of
 // memory latency for 22 MB.  Sums are kept as hi + lo, the error-free transformation of each addition
 // (Knuth's TwoSum), to about 48 bits like FP64 would, at FP32 rate.
@@ -892,12 +892,12 @@ wgrad_reduce(const float* part, int nparts, int cout, int cin, float* dW, float*
             const int dtp = tap / 9, dhp = (tap / 3) % 3;
             dw = tap % 3;
             n = (2 - dtp) * NCO * 8 + co;
-            m = dhp * 32 + ci;
+            m = dhp * C::XC + ci;
         } else {
             const int co = idx - total;
             dw = 1;
             n = NCO * 8 + co;
-            m = 96;
+            m = 3 * C::XC;
         }
         const float* p0 = part + ((size_t)dw * C::N + n) * 128 + m;
 #pragma unroll 4
@@ -1067,32 +1067,18 @@ EncodeFn encode() {
     return fn;
 }
 
-// 4D map over a channels-last bf16 activation [T][H][W][C], C = 16 or 32; box = all channels x 130
-// voxels x 1 row x `frames`, each voxel's 32 or 64 bytes swizzled (the A operand's rows).
-bool act_map(CUtensorMap* m, const void* base, int C, int T, int H, int W, int frames) {
+// 4D map over a channels-last bf16 activation [T][H][W][C], C = 16 or 32; box = all channels x `vox`
+// voxels x `rows` rows x `frames`, each voxel's 32 or 64 bytes swizzled.
+bool act_map(CUtensorMap* m, const void* base, int C, int T, int H, int W, int vox, int rows, int frames) {
     EncodeFn fn = encode();
     if (!fn) return false;
     cuuint64_t dims[4] = {(cuuint64_t)C, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)T};
     cuuint64_t str[3] = {(cuuint64_t)C * 2, (cuuint64_t)C * 2 * W, (cuuint64_t)C * 2 * W * H};
-    cuuint32_t box[4] = {(cuuint32_t)C, (cuuint32_t)RW, 1, (cuuint32_t)frames};
+    cuuint32_t box[4] = {(cuuint32_t)C, (cuuint32_t)vox, (cuuint32_t)rows, (cuuint32_t)frames};
     cuuint32_t es[4] = {1, 1, 1, 1};
     return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, str, box, es,
               CU_TENSOR_MAP_INTERLEAVE_NONE, C == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_32B,
               CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
-// 4D map over a channels-last bf16 activation [T][H][W][C] with a box of 8 channels x bw voxels
-// x 1 row x 1 frame (one chunk of one row).
-bool row_map(CUtensorMap* m, const void* base, int C, int T, int H, int W, int bw) {
-    EncodeFn fn = encode();
-    if (!fn) return false;
-    cuuint64_t dims[4] = {(cuuint64_t)C, (cuuint64_t)W, (cuuint64_t)H, (cuuint64_t)T};
-    cuuint64_t str[3] = {(cuuint64_t)C * 2, (cuuint64_t)C * 2 * W, (cuuint64_t)C * 2 * W * H};
-    cuuint32_t box[4] = {8, (cuuint32_t)bw, 1, 1};
-    cuuint32_t es[4] = {1, 1, 1, 1};
-    return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims, str, box, es,
-              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
 int blocks_for(int64_t n, int per = 256) {
@@ -1175,7 +1161,7 @@ template <int CIN, int COUT, int EPI, int FR>
 int launch_conv(const void* in, int T, int H, int W, const ConvArgs& a, int items, cudaStream_t s) {
     using Cf = ConvCfg<CIN, COUT, FR>;
     CUtensorMap m;
-    if (!act_map(&m, in, CIN, T, H, W, Cf::NF)) return nfail(SFSEG_ERR_CUDA, "tensor map encoding failed");
+    if (!act_map(&m, in, CIN, T, H, W, RW, 1, Cf::NF)) return nfail(SFSEG_ERR_CUDA, "tensor map encoding failed");
     auto k = conv3d_tc<CIN, COUT, EPI, FR>;
     static unsigned long long attr_set = 0;   // devices on which the attribute is set
     if (!(attr_set & device_bit())) {
@@ -1223,7 +1209,7 @@ template <int FR>
 int launch_last(const __nv_bfloat16* in, int T, int H, int W, const LastArgs& a, int items, cudaStream_t s) {
     using L = LastCfg<FR>;
     CUtensorMap m;
-    if (!act_map(&m, in, 32, T, H, W, L::NF)) return nfail(SFSEG_ERR_CUDA, "tensor map encoding failed");
+    if (!act_map(&m, in, 32, T, H, W, RW, 1, L::NF)) return nfail(SFSEG_ERR_CUDA, "tensor map encoding failed");
     static unsigned long long attr_set = 0;   // devices on which the attribute is set
     if (!(attr_set & device_bit())) {
         NET_CUDA(cudaFuncSetAttribute(conv_last_tc<FR>, cudaFuncAttributeMaxDynamicSharedMemorySize, L::SMEM));
@@ -1333,7 +1319,7 @@ int run_wgrad(sfseg_net* n, int cout, int cin, const __nv_bfloat16* dz, const __
               float* dW, float* db, cudaStream_t s) {
     using Cf = WgCfg<NCI, NCO>;
     CUtensorMap xm, dm;
-    if (!row_map(&xm, x, NCI * 8, T, H, W, WG_XV) || !row_map(&dm, dz, NCO * 8, T, H, W, MT))
+    if (!act_map(&xm, x, NCI * 8, T, H, W, WG_XV, 3, 1) || !act_map(&dm, dz, NCO * 8, T, H, W, MT, 1, 3))
         return nfail(SFSEG_ERR_CUDA, "tensor map encoding failed");
     if (!n->wg_part) NET_CUDA(cudaMalloc(&n->wg_part, (size_t)num_sms() * WgCfg<4, 4>::PART * sizeof(float)));
     auto k = wgrad_tc<NCI, NCO>;
