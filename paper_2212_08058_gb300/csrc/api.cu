@@ -470,6 +470,7 @@ int sfseg_power_iterate(sfseg_handle* h, const void* features, int dtype, const 
         launch_prologue(init, x_inout, h->f32, p, h->g, h->vbuf[0], vt0, record ? h->ckpt[0] : nullptr,
                         iters == 0 ? x_inout : nullptr, acc, st, s32);
         SFSEG_LAUNCHED();
+        const float* x_internal = nullptr;   // x~_iters where the last step left it, if not in x_inout
         cudaEvent_t ev0 = nullptr, ev1 = nullptr;
         if (h->timing && iters > 0) {
             ev0 = take_event(h);
@@ -486,8 +487,11 @@ int sfseg_power_iterate(sfseg_handle* h, const void* features, int dtype, const 
                 if (last) ck = last_ckpt;
                 else if ((k + 1) % record_every == 0) ck = h->ckpt[(k + 1) / record_every];
             }
-            launch_iterate(h->vbuf[k & 1], vin_t, last ? (void*)x_inout : h->vbuf[(k + 1) & 1], out_t, last, fptr,
-                           vin_t, ck, h->g, tp, inv_alpha, p, acc + k, acc + k + 1, h->flags, st, s32);
+            // the last step may leave x~ in its record or in the idle iterate buffer
+            float* xt = !last ? nullptr : (ck ? ck : (float*)h->vbuf[(k + 1) & 1]);
+            if (launch_iterate(h->vbuf[k & 1], vin_t, last ? (void*)x_inout : h->vbuf[(k + 1) & 1], out_t, last, fptr,
+                               vin_t, ck, h->g, tp, inv_alpha, p, acc + k, acc + k + 1, h->flags, st, s32, xt))
+                x_internal = xt;
             SFSEG_LAUNCHED();
         }
         if (ev1) {
@@ -495,7 +499,8 @@ int sfseg_power_iterate(sfseg_handle* h, const void* features, int dtype, const 
             h->ev_pending.emplace_back(ev0, ev1);
             h->timed_launches += iters;
         }
-        launch_scale_inv_norm(x_inout, h->N, acc + iters, h->flags, st);
+        if (x_internal) launch_scale_out(x_internal, h->g, x_inout, acc + iters, h->flags, st);
+        else launch_scale_inv_norm(x_inout, h->N, acc + iters, h->flags, st);
         SFSEG_LAUNCHED();
         return SFSEG_OK;
     };

@@ -207,7 +207,8 @@ __device__ __forceinline__ bool run_of(const Params& P, int s, Run& r) {
 // (G*(g^2 v)); it adds t = s g^{3j} (c_{3j} G*v + g (c_{3j+1} G*(g v) + g c_{3j+2} G*(g^2 v))) to out
 // (writes it when j = 0).  All in the internal layout.  MODE 8 writes x~ in the
 // internal layout and adds the largest of its outputs to P.maxkey (atomicMax of the order key, one per
-// warp): the maximum a soft-binarisation step (Alg. 1 step 3) scales by, without a pass of its own.
+// warp; nullable): the maximum a soft-binarisation step (Alg. 1 step 3) scales by, without a pass of its
+// own.  The last step of a power iteration is one too, without the key.
 template <int RT, int RH, int RW, typename TS, typename TVO, bool OUT_X, bool SEP, int MODE>
 __global__ void __launch_bounds__(NTHR, 1)
 iter_stream(const __grid_constant__ Maps M, const __grid_constant__ Params P) {
@@ -580,7 +581,7 @@ iter_stream(const __grid_constant__ Maps M, const __grid_constant__ Params P) {
         red[i] = (double)part.x + (double)part.y;
         if constexpr (MODE == 8) {
             const unsigned kmax = __reduce_max_sync(0xffffffffu, order_key(tmax));
-            if (lane == 0) atomicMax(P.maxkey, kmax);
+            if (lane == 0 && P.maxkey) atomicMax(P.maxkey, kmax);
         }
     }
     if (!ok) atomicOr(P.flags, kFlagTimeout);

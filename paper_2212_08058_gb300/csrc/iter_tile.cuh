@@ -427,7 +427,7 @@ iter_tile(const __grid_constant__ CUtensorMap mv, const __grid_constant__ CUtens
         if (tid == 0) {
             unsigned m = wmax[0];
             for (int i = 1; i < NTHR / 32; ++i) m = max(m, wmax[i]);
-            atomicMax(P.maxkey, m);
+            if (P.maxkey) atomicMax(P.maxkey, m);
         }
     }
 }

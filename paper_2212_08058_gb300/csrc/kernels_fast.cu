@@ -136,6 +136,12 @@ bool launch_iterate_fast_max(const float* vin, float* y, const float* f, const G
     return run(a);
 }
 
+bool launch_iterate_fast_last(const float* vin, float* x, const float* f, const Geom& g, const Taps& tp,
+                              float inv_alpha, float p, const double* acc_in, double* acc_out, int* flags,
+                              cudaStream_t s) {
+    return run(args(kStepMax, vin, x, f, g, tp, inv_alpha, p, acc_in, acc_out, flags, s));
+}
+
 bool launch_iterate_fast_ckpt(const float* vin, void* out, bool out_x, const float* f, const Geom& g, const Taps& tp,
                               float inv_alpha, float p, const double* acc_in, double* acc_out, float* ckpt, int* flags,
                               cudaStream_t s) {

@@ -163,22 +163,30 @@ static void iterate_t(const void* vin, void* out, const void* f, float* ckpt, Ge
     run_stencil(op, tp, 16, acc_in, acc_out, nullptr, flags, s);
 }
 
-void launch_iterate(const void* vin, int vin_type, void* out, int out_type, bool out_x, const void* f,
+bool launch_iterate(const void* vin, int vin_type, void* out, int out_type, bool out_x, const void* f,
                     int f_type, float* ckpt, Geom g, const Taps& tp, float inv_alpha, float p,
-                    const double* acc_in, double* acc_out, int* flags, cudaStream_t s, const float* s32) {
+                    const double* acc_in, double* acc_out, int* flags, cudaStream_t s, const float* s32,
+                    float* last_xt) {
     using bf = __nv_bfloat16;
+    // The last step into the internal layout; a recording one's record is that same volume.
+    if (out_x && last_xt && vin_type == kF32 && s32 == nullptr && fast_step_supported(tp) &&
+        launch_iterate_fast_last((const float*)vin, last_xt, (const float*)f, g, tp, inv_alpha, p, acc_in, acc_out,
+                                 flags, s)) {
+        note_step(true, tp, vin_type, out_type, out_x, ckpt != nullptr, false);
+        return true;
+    }
     // The TMA kernel serves the method's radii, recording steps (float32, shared maps) included.
     if (ckpt == nullptr && fast_step_supported(tp) &&
         launch_iterate_fast(vin, vin_type, out, out_type, out_x, f, g, tp, inv_alpha, p, acc_in, acc_out, flags, s,
                             s32)) {
         note_step(true, tp, vin_type, out_type, out_x, false, s32 != nullptr);
-        return;
+        return false;
     }
     if (ckpt != nullptr && vin_type == kF32 && s32 == nullptr && fast_step_supported(tp) &&
         launch_iterate_fast_ckpt((const float*)vin, out, out_x, (const float*)f, g, tp, inv_alpha, p, acc_in, acc_out,
                                  ckpt, flags, s)) {
         note_step(true, tp, vin_type, out_type, out_x, true, false);
-        return;
+        return false;
     }
     // Radii without a TMA kernel, or a tensor map the driver would not encode: the generic
     // streaming stencil (same results, slower); counted so that callers can tell.
@@ -197,6 +205,7 @@ void launch_iterate(const void* vin, int vin_type, void* out, int out_type, bool
         else SFSEG_IT(bf, float, bf, false);
     }
 #undef SFSEG_IT
+    return false;
 }
 
 void launch_apply(const float* x, int x_pitch, float* y, int y_pitch, const float* f32, Geom g,
@@ -391,6 +400,23 @@ void launch_scale_inv_norm(float* x, int64_t n, const double* acc, int* flags, c
     int blocks = (int)((n + 255) / 256);
     if (blocks > 8 * num_sms()) blocks = 8 * num_sms();
     scale_inv_norm_kernel<<<blocks, 256, 0, s>>>(x, n, aligned16(x), acc, flags); count_launches(1);
+}
+
+__global__ void scale_out_kernel(const float* xt, Geom g, float* x, bool pairs, const double* acc, int* flags) {
+    const float s = block_inv_norm(acc, flags);
+    for_each_voxel_pairs(
+        g, pairs,
+        [&](int64_t i, int64_t j) {
+            const float2 v = ld2(xt + j);
+            st2(x + i, make_float2(s * v.x, s * v.y));
+        },
+        [&](int64_t i, int64_t j) { x[i] = s * xt[j]; });
+}
+
+void launch_scale_out(const float* xt, Geom g, float* x, const double* acc, int* flags, cudaStream_t s) {
+    const RowLaunch rl = row_launch(g, num_sms(), 8);
+    scale_out_kernel<<<rl.blocks, rl.threads, 0, s>>>(xt, g, x, g.W % 2 == 0 && aligned8(x), acc, flags);
+    count_launches(1);
 }
 
 __global__ void dot2_kernel(const float* x, const float* y, int64_t n, bool vec, double* acc) {

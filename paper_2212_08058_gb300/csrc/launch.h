@@ -31,10 +31,13 @@ void launch_prologue(int init, const float* x_user, const float* f32, float p, G
 // input v_k = u x~_k (internal), output v_{k+1} = u x~_{k+1} or, when `out_x`, x~_{k+1} itself
 // in the caller's layout (pitch W).  acc_in = ||x~_k||^2, acc_out += ||x~_{k+1}||^2.
 // `ckpt` (nullable) receives an FP32 copy of x~_{k+1} in internal layout.
-void launch_iterate(const void* vin, int vin_type, void* out, int out_type, bool out_x,
+//
+// `last_xt` (nullable, an internal-layout volume other than vin): where the last step (out_x) may leave
+// x~_{k+1} instead of `out`; returns true when it did.
+bool launch_iterate(const void* vin, int vin_type, void* out, int out_type, bool out_x,
                     const void* f, int f_type, float* ckpt, Geom g, const Taps& tp,
                     float inv_alpha, float p, const double* acc_in, double* acc_out, int* flags,
-                    cudaStream_t s, const float* s32 = nullptr);
+                    cudaStream_t s, const float* s32 = nullptr, float* last_xt = nullptr);
 
 // TMA-staged step for the radii with a compiled kernel (kernels_fast.cu).  s32
 // (nullable): a separate unary map (float32 storage only).  Returns false when the radius has no
@@ -52,6 +55,13 @@ bool launch_iterate_fast(const void* vin, int vin_type, void* out, int out_type,
 // launched) for a radius without a compiled kernel.
 bool launch_iterate_fast_max(const float* vin, float* y, const float* f, const Geom& g, const Taps& tp,
                              float inv_alpha, float p, unsigned* maxkey, int* flags, cudaStream_t s);
+
+// The last step of a power iteration, float32 and shared maps: x~_{k+1} in the internal layout (the scale
+// pass converts it: the step's own stores to a caller's rows of any alignment cost 10 % of the launch).
+// False (nothing launched) for a radius that no compiled kernel covers.
+bool launch_iterate_fast_last(const float* vin, float* x, const float* f, const Geom& g, const Taps& tp,
+                              float inv_alpha, float p, const double* acc_in, double* acc_out, int* flags,
+                              cudaStream_t s);
 
 // v = u x (internal layout) for a caller-layout x, u = s^p with s the unary map (s32, or f32).
 void launch_to_state(const float* x, const float* f32, const float* s32, float p, Geom g, float* v, cudaStream_t s);
@@ -151,6 +161,9 @@ int handle_push_frame(sfseg_handle* h, const void* frame, int dtype, const float
 // Bounded-wait self-test (selftest.cu): waits `spins` times on an mbarrier nothing completes,
 // then raises kFlagTimeout.
 void launch_wait_probe(long long spins, int* flags, cudaStream_t s);
+
+// x = xt / sqrt(*acc), xt in the internal layout, x in the caller's.
+void launch_scale_out(const float* xt, Geom g, float* x, const double* acc, int* flags, cudaStream_t s);
 
 // x *= 1/sqrt(*acc) over a caller-layout volume.
 void launch_scale_inv_norm(float* x, int64_t n, const double* acc, int* flags, cudaStream_t s);

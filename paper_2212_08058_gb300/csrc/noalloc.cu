@@ -117,12 +117,15 @@ extern "C" int sfseg_power_iterate_noalloc(const sfseg_params* prm, int C, int T
     const float inv_alpha = (float)(1.0 / prm->alpha), p = (float)prm->p;
     launch_combine(features, dtype, C, g, wdev, bias, f32, nullptr, flags, s);
     launch_prologue(init, x_inout, f32, p, g, vbuf[0], kF32, nullptr, iters == 0 ? x_inout : nullptr, acc, s);
+    bool internal = false;
     for (int k = 0; k < iters; ++k) {
         const bool last = k == iters - 1;
-        launch_iterate(vbuf[k & 1], kF32, last ? (void*)x_inout : vbuf[(k + 1) & 1], kF32, last, f32, kF32, nullptr,
-                       g, tp, inv_alpha, p, acc + k, acc + k + 1, flags, s);
+        internal = launch_iterate(vbuf[k & 1], kF32, last ? (void*)x_inout : vbuf[(k + 1) & 1], kF32, last, f32, kF32, nullptr,
+                       g, tp, inv_alpha, p, acc + k, acc + k + 1, flags, s, nullptr,
+                       last ? (float*)vbuf[(k + 1) & 1] : nullptr);
     }
-    launch_scale_inv_norm(x_inout, N, acc + iters, flags, s);
+    if (internal) launch_scale_out((const float*)vbuf[iters & 1], g, x_inout, acc + iters, flags, s);
+    else launch_scale_inv_norm(x_inout, N, acc + iters, flags, s);
     if ((e = cudaGetLastError()) != cudaSuccess)
         return fail(SFSEG_ERR_CUDA, std::string("kernel launch: ") + cudaGetErrorString(e));
     if (norms_out) {
