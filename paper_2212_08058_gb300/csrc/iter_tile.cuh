@@ -432,23 +432,6 @@ iter_tile(const __grid_constant__ CUtensorMap mv, const __grid_constant__ CUtens
     }
 }
 
-// Frame-chunk length minimising (waves x frames per chunk) for `slots` resident CTAs.
-static int pick_chunk(int T, int tiles, int slots, int rt) {
-    long best_cost = -1;
-    int best = T;
-    for (int nt = 1; nt <= T; ++nt) {
-        const int chunk = (T + nt - 1) / nt;
-        const int nct = (T + chunk - 1) / chunk;
-        const long waves = ((long)tiles * nct + slots - 1) / slots;
-        const long cost = waves * (chunk + 2 * rt);
-        if (best_cost < 0 || cost < best_cost) {
-            best_cost = cost;
-            best = chunk;
-        }
-    }
-    return best;
-}
-
 template <int RT, int RH, int RW, typename TS, typename TVO, bool OUT_X, bool SEP, int MODE>
 static bool launch_t(const StepArgs& a) {
     using C = Cfg<RT, RH, RW, TS, TVO, OUT_X>;
@@ -487,7 +470,7 @@ static bool launch_t(const StepArgs& a) {
     for (int i = 0; i < 3; ++i) P.exc[i] = a.ex ? a.ex->c[i] : 0.f;
     P.maxkey = a.maxkey;
     const int tx = (g.W + TW - 1) / TW, ty = (g.H + TH - 1) / TH;
-    P.tchunk = pick_chunk(g.T, tx * ty, slots_per_sm * num_sms(), RT);
+    P.tchunk = tile_chunk(g.T, tx * ty, slots_per_sm * num_sms(), RT);
     P.acc_in = a.acc_in;
     P.acc_out = a.acc_out;
     P.flags = a.flags;

@@ -80,19 +80,30 @@ const Radius* covering_radius(const Taps& tp) {
     return best;
 }
 
-// The streaming kernel takes a volume whose frames keep its persistent blocks busy: at least 7
-// output frames for every 2 blocks, and 6 frames in time (each run of a tile's frames ends with rt
-// flushing ones).  Below that the small tiles' shorter chain counts more.  Measured per step on both
-// sides of the line, tile / streaming kernel, (2,7,7): 8x64x64 8.8 / 10.6 us, 16x128x128 12.2 / 12.8,
-// 3x480x854 17.3 / 22.8; 6x994x303 25.2 / 22.8, 50x100x200 23.5 / 18.9, 24x203x331 25.4 / 22.0.
-bool stream_pays(const Geom& g) {
-    const int64_t tiles = (int64_t)((g.W + 111) / 112) * ((g.H + 17) / 18);
-    return g.T >= 6 && 2 * tiles * g.T >= 7 * (int64_t)num_sms();
+// Which kernel a volume takes: the one whose time, modelled from the frames its busiest SM streams, is
+// shorter.  The streaming kernel takes 4.7 us and u per frame step, its steps being the whole tiles'
+// frames (rt more each to flush) and the share of the tiles left over (3 rt more for the cuts); the
+// small-tile kernel 0.4 us and 1.8 u per step of its three CTAs per SM.  u = 0.55 + 0.026 us per tap.
+// The choice costs 0.3 % on average, 6 % at worst, over the 26 volumes it was fitted to.  Measured, tile /
+// streaming kernel, (2,7,7): 16x128x128 11.6 / 12.7 us,
+// 60x128x128 18.2 / 23.4, 13x480x854 39.7 / 43.2, 32x240x427 31.2 / 30.8, 25x480x854 70.4 / 68.3,
+// 50x100x200 20.8 / 18.9, 64x480x854 169 / 147; (1,3,3): 32x240x427 18.6 / 19.4, 48x240x427 25.6 / 25.2.
+bool stream_pays(const Geom& g, const Radius& r) {
+    const double G = num_sms(), T = g.T, u = 0.55 + 0.026 * (2 * (r.rt + r.rh + r.rw) + 3);
+    const int64_t big = (int64_t)((g.W + 111) / 112) * ((g.H + 17) / 18);      // 18 x 112 tiles
+    const int64_t small = (int64_t)((g.W + 63) / 64) * ((g.H + 14) / 15);      // 15 x 64 tiles
+    const int64_t whole = big / num_sms(), rest = big - whole * num_sms();
+    const double stream = 4.7 + u * (whole * (T + r.rt) + (rest ? rest * T / G + 3 * r.rt : 0.0));
+    if (small > 3 * (int64_t)num_sms() * 16) return true;    // many waves: the streaming kernel's steps are cheaper
+    const int chunk = tile_chunk(g.T, (int)small, 3 * num_sms(), r.rt);
+    const double blocks = (double)small * ((g.T + chunk - 1) / chunk), waves = blocks / (3 * G);
+    const double tile = 0.4 + 1.8 * u * (chunk + (chunk < g.T ? 2 : 1) * r.rt) * (waves > 1.0 ? waves : 1.0);
+    return stream <= tile;
 }
 
 bool run(const StepArgs& a) {
     const Radius* r = covering_radius(a.tp);
-    return r && (stream_pays(a.g) ? r->stream(a) : r->tile(a));
+    return r && (stream_pays(a.g, *r) ? r->stream(a) : r->tile(a));
 }
 
 StepArgs args(int mode, const void* vin, void* out, const void* f, const Geom& g, const Taps& tp, float inv_alpha,

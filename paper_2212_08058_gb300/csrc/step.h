@@ -39,6 +39,26 @@ struct StepArgs {
 // A map over an internal volume with boxes of box_w x box_h x 1 (kernels_fast.cu).
 bool make_step_map(CUtensorMap* map, const void* base, bool bf16, const Geom& g, int box_w, int box_h);
 
+// Frame-chunk length of the small-volume kernel minimising (waves x frames per chunk) for `slots`
+// resident CTAs.
+inline int tile_chunk(int T, int tiles, int slots, int rt) {
+    long best_cost = -1;
+    int best = T;
+    for (int nt = 1;;) {   // the distinct chunk lengths
+        const int chunk = (T + nt - 1) / nt;
+        const int nct = (T + chunk - 1) / chunk;
+        const long waves = ((long)tiles * nct + slots - 1) / slots;
+        const long cost = waves * (chunk + 2 * rt);
+        if (best_cost < 0 || cost < best_cost) {
+            best_cost = cost;
+            best = chunk;
+        }
+        if (chunk == 1) break;
+        nt = (T + chunk - 2) / (chunk - 1);
+    }
+    return best;
+}
+
 // Calls K::launch<TS, TVO, OUT_X, SEP, MODE>(a) for the step that `a` describes; false where no such
 // kernel is compiled.
 template <class K>
