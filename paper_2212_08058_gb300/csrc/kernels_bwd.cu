@@ -19,6 +19,7 @@
 #include "common.cuh"
 #include "launch.h"
 #include "stencil.cuh"
+#include "tma.cuh"
 #include "voxels.cuh"
 
 namespace sfseg {
@@ -134,6 +135,7 @@ void launch_adjoint_first(const float* xK, const double* accK, const float* gK, 
 __global__ void adjoint_combine_state_kernel(const float* f, const float* vg, const float* qx, const float* Vk,
                                              const float* qg, const float* Gk, const double* acc_k,
                                              const double* dsum, Geom g, float* gz, float* vg_next) {
+    wait_previous_grid();
     const float sk = block_inv_norm<0>(acc_k, nullptr);
     const float dot = sk * block_value<1>([&] { return (float)*dsum; });
     // rows (t, h) over the blocks, four columns per thread (internal rows start 128-byte
@@ -179,7 +181,8 @@ void launch_adjoint_combine_state(const float* f32, const float* vg, const float
     const int64_t rows = (int64_t)g.T * g.H;
     const int64_t cap = (int64_t)16 * num_sms();
     const int blocks = (int)(rows < cap ? (rows > 0 ? rows : 1) : cap);
-    adjoint_combine_state_kernel<<<blocks, threads, 0, s>>>(f32, vg, qx, Vk, qg, Gk, acc_k, dsum, g, gz, vg_next);
+    launch_after_previous(adjoint_combine_state_kernel, dim3(blocks), threads, 0, s, f32, vg, qx, Vk, qg, Gk, acc_k,
+                          dsum, g, gz, vg_next);
     count_launches(1);
 }
 

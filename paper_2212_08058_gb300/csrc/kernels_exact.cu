@@ -14,6 +14,7 @@
 // 1449 us with the series in f, 659 us now.
 #include "launch.h"
 #include "order_key.cuh"
+#include "tma.cuh"
 #include "voxels.cuh"
 
 namespace sfseg {
@@ -81,6 +82,7 @@ __global__ void exact_in_kernel(const float* x_user, const float* A, Geom g, flo
 }
 
 __global__ void exact_mid_kernel(const float* S, const float* A, float inv_alpha, Geom g, float* w, double* acc) {
+    wait_previous_grid();
     float part = 0.f;
     auto one = [&](float s, float a) {
         const float x = a * s * inv_alpha;
@@ -98,6 +100,7 @@ __global__ void exact_mid_kernel(const float* S, const float* A, float inv_alpha
 }
 
 __global__ void exact_next_kernel(const float* gf, Geom g, float* v) {
+    wait_previous_grid();
     for_each_quad(
         g,
         [&](int64_t j) {
@@ -139,13 +142,13 @@ void launch_exact_in(const float* x_user, const float* A, Geom g, float* w, doub
 
 void launch_exact_mid(const float* S, const float* A, float inv_alpha, Geom g, float* w, double* acc, cudaStream_t s) {
     const RowLaunch rl = quad_launch(g, 16);
-    exact_mid_kernel<<<rl.blocks, rl.threads, 0, s>>>(S, A, inv_alpha, g, w, acc);
+    launch_after_previous(exact_mid_kernel, dim3(rl.blocks), rl.threads, 0, s, S, A, inv_alpha, g, w, acc);
     count_launches(1);
 }
 
 void launch_exact_next(const float* gf, Geom g, float* v, cudaStream_t s) {
     const RowLaunch rl = quad_launch(g, 16);
-    exact_next_kernel<<<rl.blocks, rl.threads, 0, s>>>(gf, g, v);
+    launch_after_previous(exact_next_kernel, dim3(rl.blocks), rl.threads, 0, s, gf, g, v);
     count_launches(1);
 }
 

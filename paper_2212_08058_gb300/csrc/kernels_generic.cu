@@ -22,6 +22,7 @@
 #include "common.cuh"
 #include "launch.h"
 #include "stencil.cuh"
+#include "tma.cuh"
 #include "voxels.cuh"
 
 namespace sfseg {
@@ -403,6 +404,7 @@ void launch_scale_inv_norm(float* x, int64_t n, const double* acc, int* flags, c
 }
 
 __global__ void scale_out_kernel(const float* xt, Geom g, float* x, bool pairs, const double* acc, int* flags) {
+    wait_previous_grid();
     const float s = block_inv_norm(acc, flags);
     for_each_voxel_pairs(
         g, pairs,
@@ -415,7 +417,8 @@ __global__ void scale_out_kernel(const float* xt, Geom g, float* x, bool pairs, 
 
 void launch_scale_out(const float* xt, Geom g, float* x, const double* acc, int* flags, cudaStream_t s) {
     const RowLaunch rl = row_launch(g, num_sms(), 8);
-    scale_out_kernel<<<rl.blocks, rl.threads, 0, s>>>(xt, g, x, g.W % 2 == 0 && aligned8(x), acc, flags);
+    launch_after_previous(scale_out_kernel, dim3(rl.blocks), rl.threads, 0, s, xt, g, x, g.W % 2 == 0 && aligned8(x), acc,
+                          flags);
     count_launches(1);
 }
 

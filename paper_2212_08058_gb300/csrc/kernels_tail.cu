@@ -13,6 +13,7 @@
 #include "common.cuh"
 #include "launch.h"
 #include "order_key.cuh"
+#include "tma.cuh"
 #include "voxels.cuh"
 
 namespace sfseg {
@@ -41,6 +42,7 @@ __global__ void max_key_kernel(const float* y, int64_t n, unsigned* key) {
 template <bool YI>
 __global__ void sigmoid_step_kernel(const float* y, const unsigned* key, float gain, float center, const float* sm,
                                     float p, Geom g, float* x, float* v, unsigned char* mask, int* flags) {
+    wait_previous_grid();
     const float m = order_value(*key);
     if (!(m > 0.f) || isinf(m)) {
         if (blockIdx.x == 0 && threadIdx.x == 0)
@@ -93,9 +95,11 @@ void launch_sigmoid_step(const float* y, bool y_internal, const unsigned* key, f
     RowLaunch rl = row_launch(g, num_sms());
     if (y_internal) {
         if (!x && !mask) rl.threads = g.W >= 512 ? 128 : (((g.W + 3) / 4 + 31) / 32) * 32;
-        sigmoid_step_kernel<true><<<rl.blocks, rl.threads, 0, s>>>(y, key, gain, center, sm, p, g, x, v, mask, flags);
+        launch_after_previous(sigmoid_step_kernel<true>, dim3(rl.blocks), rl.threads, 0, s, y, key, gain, center, sm, p,
+                              g, x, v, mask, flags);
     } else {
-        sigmoid_step_kernel<false><<<rl.blocks, rl.threads, 0, s>>>(y, key, gain, center, sm, p, g, x, v, mask, flags);
+        launch_after_previous(sigmoid_step_kernel<false>, dim3(rl.blocks), rl.threads, 0, s, y, key, gain, center, sm, p,
+                              g, x, v, mask, flags);
     }
     count_launches(1);
 }

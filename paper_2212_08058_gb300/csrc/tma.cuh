@@ -73,7 +73,7 @@ __device__ __forceinline__ void allow_next_grid() { asm volatile("griddepcontrol
 
 // Launches `kern` as a programmatic dependent of the launch before it in the stream (the kernel
 // calls wait_previous_grid).  A failed launch is left for the caller's cudaGetLastError, as with
-// <<<>>>.
+// <<<>>>.  The arguments are converted to the kernel's parameter types.
 template <typename... KArgs, typename... Args>
 inline void launch_after_previous(void (*kern)(KArgs...), dim3 grid, int threads, int smem, cudaStream_t s,
                                   const Args&... args) {
@@ -87,7 +87,7 @@ inline void launch_after_previous(void (*kern)(KArgs...), dim3 grid, int threads
     lc.stream = s;
     lc.attrs = &at;
     lc.numAttrs = 1;
-    (void)cudaLaunchKernelEx(&lc, kern, args...);
+    (void)cudaLaunchKernelEx(&lc, kern, static_cast<const KArgs&>(args)...);
 }
 
 }  // namespace sfseg
