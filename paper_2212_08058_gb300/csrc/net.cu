@@ -35,6 +35,7 @@
 #include "../../include/sfseg.h"
 #include "common.cuh"
 #include "launch.h"
+#include "tma.cuh"
 #include "voxels.cuh"
 
 namespace sfseg {
@@ -289,8 +290,10 @@ conv3d_tc(const __grid_constant__ CUtensorMap xin, ConvArgs a) {
         tmem_st_wait();
     }
     tc_fence_before();
+    allow_next_grid();
     __syncthreads();
     tc_fence_after();
+    wait_previous_grid();            // nothing above reads or writes global memory
 
     int issued = 0;                  // producer: input rows requested so far
     if (warp == 0) {
@@ -553,6 +556,8 @@ conv_last_tc(const __grid_constant__ CUtensorMap xin, LastArgs a) {
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
+    allow_next_grid();
+    wait_previous_grid();            // nothing above reads or writes global memory
 
     int issued = 0;
     if (warp == 0) {
@@ -778,6 +783,8 @@ wgrad_tc(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUten
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
+    allow_next_grid();
+    wait_previous_grid();            // nothing above reads or writes global memory
 
     int issued = 0;
     bool mma_ok = true;
@@ -881,6 +888,7 @@ __global__ void __launch_bounds__(32 * kRedWarps)
 wgrad_reduce(const float* part, int nparts, int cout, int cin, float* dW, float* db) {
     using C = WgCfg<NCI, NCO>;
     __shared__ TwoFloat sums[kRedWarps][32];
+    wait_previous_grid();
     const int total = cout * 27 * cin;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int idx = blockIdx.x * 32 + lane;
@@ -1168,7 +1176,7 @@ int launch_conv(const void* in, int T, int H, int W, const ConvArgs& a, int item
         NET_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, Cf::SMEM));
         attr_set |= device_bit();
     }
-    k<<<items, Cf::NTHR, Cf::SMEM, s>>>(m, a);
+    launch_after_previous(k, dim3(items), Cf::NTHR, Cf::SMEM, s, m, a);
     count_launches(1);
     NET_CUDA(cudaGetLastError());
     last_shape[0] = {FR, a.HR, items};
@@ -1215,7 +1223,7 @@ int launch_last(const __nv_bfloat16* in, int T, int H, int W, const LastArgs& a,
         NET_CUDA(cudaFuncSetAttribute(conv_last_tc<FR>, cudaFuncAttributeMaxDynamicSharedMemorySize, L::SMEM));
         attr_set |= device_bit();
     }
-    conv_last_tc<FR><<<items, L::NTHR, L::SMEM, s>>>(m, a);
+    launch_after_previous(conv_last_tc<FR>, dim3(items), L::NTHR, L::SMEM, s, m, a);
     count_launches(1);
     NET_CUDA(cudaGetLastError());
     last_shape[1] = {FR, a.HR, items};
@@ -1336,9 +1344,9 @@ int run_wgrad(sfseg_net* n, int cout, int cin, const __nv_bfloat16* dz, const __
     a.flags = n->flags;
     a.per = (a.units + num_sms() - 1) / num_sms();
     const int grid = (a.units + a.per - 1) / a.per;   // every CTA gets at least one unit
-    k<<<grid, NTHR, Cf::SMEM, s>>>(xm, dm, a);
-    wgrad_reduce<NCI, NCO><<<(cout * 27 * cin + cout + 31) / 32, 32 * kRedWarps, 0, s>>>(n->wg_part, grid, cout, cin,
-                                                                                        dW, db);
+    launch_after_previous(k, dim3(grid), NTHR, Cf::SMEM, s, xm, dm, a);
+    launch_after_previous(wgrad_reduce<NCI, NCO>, dim3((cout * 27 * cin + cout + 31) / 32), 32 * kRedWarps, 0, s,
+                          n->wg_part, grid, cout, cin, dW, db);
     count_launches(2);
     NET_CUDA(cudaGetLastError());
     return SFSEG_OK;
