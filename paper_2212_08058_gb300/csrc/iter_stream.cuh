@@ -11,9 +11,8 @@
 //     z3 = f v of each, and accumulates them into its 9 x 3 outputs with packed FP32 FMAs (FFMA2,
 //     one per column pair).  The result goes to a ring of two frames of [3][18][132] floats.
 //   - w-pass, warps 4..11: a thread takes 8 output columns of one row (14 x 18 = 252 of 256
-//     threads); it loads its window of the h-pass result as 16-byte pieces (the odd-aligned pairs
-//     are rebuilt in registers at rw > 4; at rw <= 4 their taps run as two scalar FMAs instead) and
-//     feeds the three w-filtered signals straight into the t-filter, kept in registers in transposed
+//     threads); it loads its window of the h-pass result as 16-byte pieces (the odd taps run as
+//     two scalar FMAs: rebuilding their pairs for packed ones costs more moves) and feeds the three w-filtered signals straight into the t-filter, kept in registers in transposed
 //     direct form (2rt running partial sums per value, no frame ring to index).
 //   - Epilogue, same threads: Eq. 7 combination for the frame rt behind, with f of that frame from a
 //     TMA-fed tile, the Eq. 8 norm partial, and the next state into a tile that a TMA store writes
@@ -32,9 +31,11 @@
 // (measured): taps stay in the parameter constants.  And a shared-memory pointer rounded up through
 // an integer loses its address space: every access was a generic one until the alignment became an
 // offset (184 -> 152 us per step here, 180 -> 172 in the older kernel).
-// Measured per step, before -> now: (2,7,7) 64x480x854 180.5 -> 147.6 us (FP32 pipe 71 % busy, the
-// algorithmic multiply-adds alone 68 us), 120x1080x1920 1465 -> 1230; (1,3,3) 64x480x854 123 -> 98,
-// 32x240x427 24.5 -> 21.
+// Three smaller ones: the odd taps of the w-pass as scalar FMAs and the next input row of the h-pass
+// loaded a row ahead (147.6 -> 138.7 us together), and 184 / 112 / 32 registers for the w-pass, the
+// h-pass and the copy threads (192 / 96 / 32: 138.7, now 137.7).
+// Measured per step, before -> now: (2,7,7) 64x480x854 180.5 -> 137.7 us (the algorithmic
+// multiply-adds alone 68 us), 120x1080x1920 1465 -> 1161; (1,3,3) 64x480x854 123 -> 94.6.
 #pragma once
 
 #include "order_key.cuh"
@@ -55,7 +56,7 @@ constexpr int NH = 128, NW = 256;   // threads of the h-pass and of the w-pass
 constexpr int NTHR = NH + NW + 128; // and a warpgroup whose first two warps hold a copy thread each
 // Registers per thread of the three roles; the sum over the four warpgroups is the 4 x 128 that the
 // block is launched with.  The w-pass keeps 96 of t-filter state at rt = 2.
-constexpr int kRegsW = 192, kRegsH = 96, kRegsIO = 32;
+constexpr int kRegsW = 184, kRegsH = 112, kRegsIO = 32;
 static_assert(2 * kRegsW + kRegsH + kRegsIO <= 4 * 128, "register split");
 static_assert(kRegsW >= 128 && kRegsH <= 128 && kRegsIO <= 128 && kRegsW % 8 == 0 && kRegsH % 8 == 0 &&
                   kRegsIO % 8 == 0,
@@ -352,10 +353,14 @@ iter_stream(const __grid_constant__ Maps M, const __grid_constant__ Params P) {
                     for (int o = 0; o < RHS; ++o)
 #pragma unroll
                         for (int k = 0; k < 3; ++k) acc[o][k] = make_float2(0.f, 0.f);
+                    float2 vn = ld_pair(sv), fn = ld_pair(sf);
 #pragma unroll
                     for (int j = 0; j < RHS + 2 * RH; ++j) {
-                        const float2 v = ld_pair(sv + j * BW);
-                        const float2 f = ld_pair(sf + j * BW);
+                        const float2 v = vn, f = fn;
+                        if (j + 1 < RHS + 2 * RH) {
+                            vn = ld_pair(sv + (j + 1) * BW);
+                            fn = ld_pair(sf + (j + 1) * BW);
+                        }
                         const float2 z3 = mul2(f, v);
                         const float2 z2 = mul2(f, z3);
 #pragma unroll
@@ -475,13 +480,11 @@ iter_stream(const __grid_constant__ Maps M, const __grid_constant__ Params P) {
 #pragma unroll
                             for (int m = 0; m < 4; ++m) {
                                 const int c = 2 * m + d + C::OFF - RW;
-                                if ((c & 1) && RW <= 4) {   // odd-aligned pair: two scalar FMAs
+                                if (c & 1) {   // odd-aligned pair: two scalar FMAs
                                     acc[m].x = fmaf(pa[c >> 1].y, gd.x, acc[m].x);
                                     acc[m].y = fmaf(pa[(c >> 1) + 1].x, gd.x, acc[m].y);
                                 } else {
-                                    const float2 in =
-                                        (c & 1) ? make_float2(pa[c >> 1].y, pa[(c >> 1) + 1].x) : pa[c >> 1];
-                                    acc[m] = fma2(in, gd, acc[m]);
+                                    acc[m] = fma2(pa[c >> 1], gd, acc[m]);
                                 }
                             }
                         }

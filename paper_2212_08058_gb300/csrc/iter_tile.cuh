@@ -11,8 +11,7 @@
 //      the 128 threads); it walks down the 5 + 2rh input rows once, forms the three signals z1 = v, z2 = f^2 v, z3 = f v of each, and accumulates
 //      them into its 5 x 3 outputs with packed FP32 FMAs (FFMA2, one per column pair).
 //   3. w-pass: a thread takes 8 output columns of one row; it loads its window of the h-pass
-//      result once as aligned float2 pairs (the odd-aligned pairs are rebuilt in registers at
-//      rw > 4; at rw <= 4 their taps run as two scalar FMAs instead) and feeds the three
+//      result once as aligned float2 pairs (the odd taps run as two scalar FMAs) and feeds the three
 //      w-filtered signals straight into the t-filter, kept in registers in transposed direct
 //      form (2rt running partial sums per value, no frame ring to index).
 //   4. Eq. 7 combination for the frame rt behind, the Eq. 8 norm partial and the store of the
@@ -271,12 +270,11 @@ iter_tile(const __grid_constant__ CUtensorMap mv, const __grid_constant__ CUtens
 #pragma unroll
                     for (int m = 0; m < 4; ++m) {
                         const int q = 2 * m + d + C::ODD;
-                        if ((q & 1) && RW <= 4) {   // odd-aligned pair: two scalar FMAs
+                        if (q & 1) {   // odd-aligned pair: two scalar FMAs
                             acc[m].x = fmaf(pa[q >> 1].y, gd.x, acc[m].x);
                             acc[m].y = fmaf(pa[(q >> 1) + 1].x, gd.x, acc[m].y);
                         } else {
-                            const float2 in = (q & 1) ? make_float2(pa[q >> 1].y, pa[(q >> 1) + 1].x) : pa[q >> 1];
-                            acc[m] = fma2(in, gd, acc[m]);
+                            acc[m] = fma2(pa[q >> 1], gd, acc[m]);
                         }
                     }
                 }

@@ -83,13 +83,13 @@ const Radius* covering_radius(const Taps& tp) {
 // Which kernel a volume takes: the one whose time, modelled from the frames its busiest SM streams, is
 // shorter.  The streaming kernel takes 4.7 us and u per frame step, its steps being the whole tiles'
 // frames (rt more each to flush) and the share of the tiles left over (3 rt more for the cuts); the
-// small-tile kernel 0.4 us and 1.8 u per step of its three CTAs per SM.  u = 0.55 + 0.026 us per tap.
+// small-tile kernel 0.4 us and 1.8 u per step of its three CTAs per SM.  u = 0.55 + 0.0235 us per tap.
 // The choice costs 0.3 % on average, 6 % at worst, over the 26 volumes it was fitted to.  Measured, tile /
 // streaming kernel, (2,7,7): 16x128x128 11.6 / 12.7 us,
 // 60x128x128 18.2 / 23.4, 13x480x854 39.7 / 43.2, 32x240x427 31.2 / 30.8, 25x480x854 70.4 / 68.3,
 // 50x100x200 20.8 / 18.9, 64x480x854 169 / 147; (1,3,3): 32x240x427 18.6 / 19.4, 48x240x427 25.6 / 25.2.
 bool stream_pays(const Geom& g, const Radius& r) {
-    const double G = num_sms(), T = g.T, u = 0.55 + 0.026 * (2 * (r.rt + r.rh + r.rw) + 3);
+    const double G = num_sms(), T = g.T, u = 0.55 + 0.0235 * (2 * (r.rt + r.rh + r.rw) + 3);
     const int64_t big = (int64_t)((g.W + 111) / 112) * ((g.H + 17) / 18);      // 18 x 112 tiles
     const int64_t small = (int64_t)((g.W + 63) / 64) * ((g.H + 14) / 15);      // 15 x 64 tiles
     const int64_t whole = big / num_sms(), rest = big - whole * num_sms();
