@@ -31,8 +31,8 @@ RADIUS = (2, 7, 7)
 ITERS = 50
 SEED = 2000
 WORKLOAD = "plain SFSeg 480p: C=1 fp32 64x480x854, three crossing blobs, radius (2,7,7), 50 iterations"
-PROFILE_FILE = os.path.join(ROOT, "profiles", "iter_fast_r277_f32_480p.txt")
-KERNEL_SOURCES = ["kernels_fast.cu", "common.cuh"]
+PROFILE_FILE = os.path.join(ROOT, "profiles", "iter_stream_r277_f32_480p.txt")
+KERNEL_SOURCES = ["iter_stream.cuh", "tma.cuh", "step.h", "common.cuh"]
 FMA_PER_VOXEL = 3 * ((2 * RADIUS[0] + 1) + (2 * RADIUS[1] + 1) + (2 * RADIUS[2] + 1))   # 105 at (2,7,7)
 
 
@@ -672,9 +672,10 @@ def bench_exact_kernel(sfseg, synth, ref_iters: int = 1500, alphas=(1.0, 0.5, 0.
                       "angle_deg": angle(xm, xe), "iou_half_max": iou(xm, xe)})
         if ai == 0:
             out["exact_ms_per_step"] = e0.elapsed_time(e1) / ref_iters
-            # series length as the library picks it (tail bound of the series below 2^-24)
-            xb = 2.0 * alpha * float(V.max().item()) ** 2
-            tail, terms = xb * np.exp(xb), 1
+            # series length as the library picks it: f centred on its range, the tail bound of the
+            # series in g = f - c relative to the sum's lower bound e^-x below 2^-24
+            xb = 2.0 * alpha * (0.5 * float(V.max().item() - V.min().item())) ** 2
+            tail, terms = xb * np.exp(2.0 * xb), 1
             while tail > 2.0 ** -24:
                 tail *= xb / (terms + 1)
                 terms += 1

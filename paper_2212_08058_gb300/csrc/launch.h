@@ -72,7 +72,7 @@ bool launch_iterate_fast_ckpt(const float* vin, void* out, bool out_x, const flo
                               float inv_alpha, float p, const double* acc_in, double* acc_out, float* ckpt, int* flags,
                               cudaStream_t s);
 
-// The adjoint's Q-pass on the TMA kernel (kernels_fast.cu, mode 1), float32, internal layout:
+// The adjoint's Q-pass on the TMA kernel (mode 1 at iter_stream), float32, internal layout:
 // for the signals c0, c1, c2 of v (G*v, G*(f^2 v), G*(f v)), writes Q = s (a1 c0 - p c1 + a3 c2)
 // to out, s = 1/sqrt(*acc_in) (or 1).  Returns false (nothing launched) for a radius that no
 // compiled kernel covers.
@@ -104,14 +104,14 @@ void launch_exact_next(const float* gf, Geom g, float* v, cudaStream_t s);
 void launch_exact_out(const float* S, const float* A, float inv_alpha, Geom g, float* x_user, double* acc,
                       cudaStream_t s);
 
-// The adjoint's recomputing step with its Q-pass (kernels_fast.cu, mode 6): from the state V_k
+// The adjoint's recomputing step with its Q-pass (mode 6 at iter_stream): from the state V_k
 // (internal layout, s = 1/sqrt(*acc_in)) writes the next state to vout exactly as the plain step
 // does, and Q = s (a1 c0 - p c1 + a3 c2) of the same filtered signals to Q.  Returns false for a
 // radius without a compiled kernel.
 bool launch_step_q_fast(const float* vin, float* vout, float* Q, const float* f, const Geom& g, const Taps& tp,
                         float inv_alpha, float p, const double* acc_in, int* flags, cudaStream_t s);
 
-// The adjoint's g-pass in state form (kernels_fast.cu, mode 5): for v_g = u g_y, writes
+// The adjoint's g-pass in state form (mode 5 at iter_stream): for v_g = u g_y, writes
 // G = u A g_y = u^2 B to G and Q (unscaled) to Qg, and adds sum V_k B to *dot (V_k = u x~_k,
 // internal layout; <x_k, A g_y> = dot / ||x~_k||).  Returns false for a radius without a
 // compiled kernel.
