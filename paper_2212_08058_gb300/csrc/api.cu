@@ -620,8 +620,16 @@ int sfseg_apply(sfseg_handle* h, const sfseg_neighborhood* nb, const float* x, f
     if (!x || !y) return fail(SFSEG_ERR_INVALID_ARG, "null x or y");
     if (x == y) return fail(SFSEG_ERR_INVALID_ARG, "x and y must not alias");
     if (!h->features_set) return fail(SFSEG_ERR_STATE, "no features set");
-    launch_apply_user(x, y, (float*)h->vbuf[1], h->f32, h->g, tp, (float)(1.0 / h->alpha), (float)h->p, h->flags,
-                      (cudaStream_t)stream, h->sep ? h->s32 : nullptr);
+    const float inv_alpha = (float)(1.0 / h->alpha), p = (float)h->p;
+    const float* s32 = h->sep ? h->s32 : nullptr;
+    // A radius padded with zero taps would carry an Inf or NaN of the caller's x past its
+    // neighbourhood (0 * Inf), so here such radii take the generic stencil.
+    if (fast_iterate_supported(tp))
+        launch_apply_user(x, y, (float*)h->vbuf[1], h->f32, h->g, tp, inv_alpha, p, h->flags, (cudaStream_t)stream,
+                          s32);
+    else
+        launch_apply(x, h->g.W, y, h->g.W, h->f32, h->g, tp, inv_alpha, p, nullptr, nullptr, h->flags,
+                     (cudaStream_t)stream, s32);
     SFSEG_LAUNCHED();
     return SFSEG_OK;
 }

@@ -86,6 +86,27 @@ def test_padded_radius_adjoint(sf, T, H, W):
     assert abs(gw[0] * d[0] + gw[1] * d[1] + gb * d[2] - num) <= 1e-4 * scale
 
 
+@pytest.mark.parametrize("radius", [(0, 0, 0), (1, 1, 1), (0, 2, 1), (1, 6, 6), (1, 3, 3)])
+def test_apply_keeps_inf_in_its_neighbourhood(sf, radius):
+    """An Inf in x reaches the outputs of its own neighbourhood and no others: those are what they are
+    with a zero in its place, bit for bit (a zero adds exactly nothing)."""
+    T, H, W = 5, 30, 40
+    g = torch.Generator(device="cuda").manual_seed(6)
+    V = torch.rand((1, T, H, W), device="cuda", generator=g) + 0.1
+    x = torch.rand((T, H, W), device="cuda", generator=g)
+    at = (2, 14, 21)
+    x[at] = 0.0
+    with sf.PowerIteration(1, T, H, W) as h:
+        h.set_features(V)
+        y0 = h.apply(x, radius).clone()
+        x[at] = float("inf")
+        y1 = h.apply(x, radius)
+    inside = torch.zeros((T, H, W), dtype=torch.bool, device="cuda")
+    inside[tuple(slice(max(c - r, 0), c + r + 1) for c, r in zip(at, radius))] = True
+    assert not torch.isfinite(y1[inside]).any()
+    assert torch.equal(y1[~inside], y0[~inside])
+
+
 def test_exact_operator_in_the_stream_kernel(sf):
     """The exact (Eq. 1) operator on a volume of the streaming kernel, with the centred series, against
     the same operator on a crop that the small-volume kernel runs, with the series in f, at voxels
