@@ -107,6 +107,19 @@ def test_apply_keeps_inf_in_its_neighbourhood(sf, radius):
     assert torch.equal(y1[~inside], y0[~inside])
 
 
+def test_norm_of_many_equal_voxels(sf):
+    """The Eq. 8 norm of a volume of 4000 tiles (26 per SM) with one feature value: a thread adds 80
+    equal squares per tile in float32, each addition 2^-24 of the sum away at most, so the root of the
+    sum 80 * 2^-25 = 2.4e-6.  One float32 sum over a thread's 26 tiles is up to 1.5e-5 away."""
+    T, H, W, r = 20, 1800, 4480, (1, 3, 3)
+    with sf.PowerIteration(1, T, H, W) as h:
+        V = torch.full((1, T, H, W), 0.6, device="cuda")
+        _, nu = h.power_iterate(V, radius=r, iters=1, return_norms=True)
+        x0 = torch.full((T, H, W), (T * H * W) ** -0.5, device="cuda")
+        y = h.apply(x0, r)
+    assert abs(float(nu[0]) / float(y.double().norm()) - 1.0) <= 2.4e-6
+
+
 def test_exact_operator_in_the_stream_kernel(sf):
     """The exact (Eq. 1) operator on a volume of the streaming kernel, with the centred series, against
     the same operator on a crop that the small-volume kernel runs, with the series in f, at voxels
