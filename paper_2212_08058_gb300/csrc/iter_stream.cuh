@@ -34,8 +34,8 @@
 // Three smaller ones: the odd taps of the w-pass as scalar FMAs and the next input row of the h-pass
 // loaded a row ahead (147.6 -> 138.7 us together), and 184 / 112 / 32 registers for the w-pass, the
 // h-pass and the copy threads (192 / 96 / 32: 138.7, now 137.7).
-// Measured per step, before -> now: (2,7,7) 64x480x854 180.5 -> 137.7 us (the algorithmic
-// multiply-adds alone 68 us), 120x1080x1920 1465 -> 1161; (1,3,3) 64x480x854 123 -> 94.6.
+// Measured per step, before -> now: (2,7,7) 64x480x854 180.5 -> 138.2 us (the algorithmic
+// multiply-adds alone 68 us), 120x1080x1920 1465 -> 1163; (1,3,3) 64x480x854 123 -> 94.6.
 #pragma once
 
 #include "order_key.cuh"
