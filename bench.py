@@ -672,10 +672,13 @@ def bench_exact_kernel(sfseg, synth, ref_iters: int = 1500, alphas=(1.0, 0.5, 0.
                       "angle_deg": angle(xm, xe), "iou_half_max": iou(xm, xe)})
         if ai == 0:
             out["exact_ms_per_step"] = e0.elapsed_time(e1) / ref_iters
-            # series length as the library picks it: f centred on its range, the tail bound of the
-            # series in g = f - c relative to the sum's lower bound e^-x below 2^-24
-            xb = 2.0 * alpha * (0.5 * float(V.max().item() - V.min().item())) ** 2
-            tail, terms = xb * np.exp(2.0 * xb), 1
+            # series length as the library picks it: f centred on its range (alpha range^2 <= 1; the
+            # tail bound in g = f - c relative to the sum's lower bound e^-x below 2^-24), else the
+            # series in f
+            lo, hi = float(V.min().item()), float(V.max().item())
+            centred = alpha * (hi - lo) ** 2 <= 1.0
+            xb = 2.0 * alpha * (0.5 * (hi - lo) if centred else hi) ** 2
+            tail, terms = xb * np.exp((2.0 if centred else 1.0) * xb), 1
             while tail > 2.0 ** -24:
                 tail *= xb / (terms + 1)
                 terms += 1

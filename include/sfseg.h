@@ -144,10 +144,12 @@ int sfseg_apply(sfseg_handle* h, const sfseg_neighborhood* nb, const float* x, f
  * in g = f - c, whose terms are separable: three terms per pass of the TMA stencil.  Shared maps only
  * (UNSUPPORTED after sfseg_set_features_sf), the radii with a TMA kernel only (UNSUPPORTED
  * otherwise), FP32 storage.  Allocates three more float32 volumes on first use.
- *   n_terms   the number of terms of the series in f (c = 0), 1..120; 0 takes c in the middle of f's
- *             range and the smallest count whose tail bound x^(N+1)/(N+1)! e^x, x = 2 alpha max(g)^2,
- *             is below 2^-24 relative to the sum (this reads f's range: the call synchronises), or
- *             returns UNSUPPORTED when 120 terms of the series in f do not reach that.
+ *   n_terms   the number of terms of the series in f (c = 0), 1..120; 0 takes the smallest count whose
+ *             tail bound x^(N+1)/(N+1)! e^x, x = 2 alpha max(g)^2, is below 2^-24 relative to the sum,
+ *             with c in the middle of f's range if alpha (max f - min f)^2 <= 1 and c = 0 otherwise
+ *             (beyond that the terms of a pair at opposite ends of the range would cancel digits of
+ *             its small weight); this reads f's range: the call synchronises.  UNSUPPORTED when 120
+ *             terms of the series in f do not reach the bound.
  *   x, y      device [T][H][W] float32 (may not alias).
  * Errors: INVALID_ARG, SHAPE, STATE (no features), UNSUPPORTED, OOM, CUDA. */
 int sfseg_apply_exact(sfseg_handle* h, const sfseg_neighborhood* nb, int n_terms, const float* x,

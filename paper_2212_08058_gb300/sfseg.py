@@ -255,7 +255,7 @@ class PowerIteration:
 
     def apply_exact(self, x: torch.Tensor, radius=(2, 7, 7), sigma=None, n_terms: int = 0) -> torch.Tensor:
         """y = (1/alpha) M x for the exact (Eq. 1) kernel (sfseg_apply_exact; n_terms = 0 picks the
-        series length from alpha and max f, which synchronises)."""
+        series length from alpha and f's range, which synchronises)."""
         self._check_volume(x, "x")
         y = torch.empty_like(x)
         _check(lib().sfseg_apply_exact(self._h, ctypes.byref(neighborhood(radius, sigma)), int(n_terms), _ptr(x),

@@ -1,5 +1,7 @@
 """GPU exact (Eq. 1) kernel, the diagnostic of the first-order approximation (Sec. 4.3), against
 the FP64 oracle's explicit Eq. 1 matrix (oracle.affinity(..., exact=True))."""
+import math
+
 import numpy as np
 import pytest
 import torch
@@ -128,3 +130,34 @@ def test_exact_errors(sf):
         with pytest.raises(sf.SFSegError) as e:
             h.power_iterate_exact((1, 3, 3), iters=2)
         assert e.value.status == "UNSUPPORTED"
+
+
+@pytest.mark.parametrize("alpha", [0.5, 1.0, 2.0, 4.0, 8.0, 12.0])
+def test_every_output_keeps_its_digits(sf, alpha):
+    """Each output's own relative error, not only the largest output's: half of the voxels at the dark
+    end of f's range and half at its bright end, the dark ones' x a millionth of the bright ones', so
+    that a dark voxel's output is a sum over pairs at opposite ends of the range, e^{-alpha} small.
+
+    Bound, in roundings of 2^-24: a series of N terms whose products g_i g_j are of one sign is a sum of
+    positive numbers, each off by the taps of the three filters, one multiplication per power of g on
+    either side (2 N), 12 for u, e^{-alpha g^2} and the combination, and 4 alpha range^2 for the rounded
+    exponents of the two exponentials.  A centre between the two ends multiplies that by e^{alpha range^2}
+    at most, which is admitted up to alpha range^2 = 1: a factor of e."""
+    T, H, W, r = 4, 20, 60, (1, 3, 3)
+    rng = np.random.default_rng(77)
+    bright = rng.random((T, H, W)) < 0.5
+    f32 = np.where(bright, rng.uniform(0.95, 1.0, (T, H, W)), rng.uniform(0.01, 0.05, (T, H, W))).astype(np.float32)
+    x = np.where(bright, 1.0, 1e-6).astype(np.float32)
+    f = f32.astype(np.float64)
+    Me = oracle.affinity(f, f, 0.1, alpha, r, exact=True)
+    yo = (Me @ x.astype(np.float64).ravel()).reshape(T, H, W) / alpha
+    with sf.PowerIteration(1, T, H, W, alpha=alpha) as h:
+        h.set_features(torch.from_numpy(f32[None]).cuda())
+        y = h.apply_exact(torch.from_numpy(x).cuda(), r).cpu().numpy().astype(np.float64)
+    q, terms = 2.0 * alpha * f.max() ** 2, 1
+    tail = q * math.exp(q)
+    while tail > 2.0 ** -24:
+        tail *= q / (terms + 1)
+        terms += 1
+    bound = (2 * sum(r) + 3 + 2 * terms + 12 + 4 * alpha) * 2.0 ** -24 * (math.e if alpha <= 1.0 else 1.0)
+    assert (np.abs(y - yo) / yo).max() <= bound
