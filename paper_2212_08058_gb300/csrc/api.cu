@@ -18,6 +18,9 @@ namespace {
 thread_local std::string g_err;
 
 int fail(int code, const std::string& msg) {
+    // An allocation that failed stays the thread's last CUDA error: without this the launch check of the
+    // next call, of any handle, would report it again.
+    if (code == SFSEG_ERR_OOM) cudaGetLastError();
     g_err = msg;
     return code;
 }
@@ -317,6 +320,7 @@ int sfseg_create(const sfseg_params* prm, int C, int T, int H, int W, sfseg_hand
     if (rc == SFSEG_OK) chk(cudaMemset(h->f32, 0, (size_t)h->NP * sizeof(float)));
     if (rc == SFSEG_OK) rc = ensure_acc(&h->acc, &h->acc_cap, 1024);
     if (rc != SFSEG_OK) {
+        cudaGetLastError();   // the allocations after the first that failed
         sfseg_destroy(h);
         return rc;
     }
