@@ -143,7 +143,8 @@ int sfseg_apply(sfseg_handle* h, const sfseg_neighborhood* nb, const float* x, f
  * series exp(-alpha (f_i - f_j)^2) = e^{-alpha g_i^2} e^{-alpha g_j^2} sum_n (2 alpha g_i g_j)^n / n!
  * in g = f - c, whose terms are separable: three terms per pass of the TMA stencil.  Shared maps only
  * (UNSUPPORTED after sfseg_set_features_sf), the radii with a TMA kernel only (UNSUPPORTED
- * otherwise), FP32 storage.  Allocates three more float32 volumes on first use.
+ * otherwise), FP32 storage.  Allocates one more float32 volume on first use, and a second one for
+ * a centred series (without the memory for it: c = 0).
  *   n_terms   the number of terms of the series in f (c = 0), 1..120; 0 takes the smallest count whose
  *             tail bound x^(N+1)/(N+1)! e^x, x = 2 alpha max(g)^2, is below 2^-24 relative to the sum,
  *             with c in the middle of f's range if alpha (max f - min f)^2 <= 1 and c = 0 otherwise

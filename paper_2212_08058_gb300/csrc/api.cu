@@ -112,8 +112,8 @@ struct sfseg_handle {
     float* adjw[3] = {nullptr, nullptr, nullptr};   // TMA-path adjoint workspace (Q_g, v_g, v_g)
     std::vector<float*> seg;
     std::vector<float*> qxs;   // TMA path: Q_x of each step of the segment being reversed
-    // the exact kernel (internal layout): the term input, g = f - c and A = u e^{-alpha g^2}
-    float *exv = nullptr, *exg = nullptr, *exa = nullptr;
+    // the exact kernel (internal layout): g = f - c (c not 0) and A = u e^{-alpha g^2}
+    float *exg = nullptr, *exa = nullptr;
     double* dots = nullptr;
     int dots_cap = 0;
     // optional CUDA-event timing of the iteration kernels
@@ -353,7 +353,6 @@ int sfseg_destroy(sfseg_handle* h) {
     cudaFree(h->gz);
     for (float* p : h->seg) cudaFree(p);
     for (float* p : h->qxs) cudaFree(p);
-    cudaFree(h->exv);
     cudaFree(h->exg);
     cudaFree(h->exa);
     cudaFree(h->dots);
@@ -664,7 +663,8 @@ constexpr double kCentredRange = 1.0;
 // The number of series terms and the centre c of g = f - c.  n_terms > 0 is the caller's choice of
 // the series in f (c = 0).  Otherwise c is the middle of f's range, which halves max |g| for f from 0 (a
 // quarter of x, and about half the terms), while the cancellation above costs no digits, else 0.  A call
-// whose series in f would be too long is refused whatever the centred one needs.
+// whose series in f would be too long is refused whatever the centred one needs, and one
+// without the memory for the volume of g takes the series in f, which reads f's own.
 int exact_terms(sfseg_handle* h, int n_terms, cudaStream_t s, int* terms_out, float* center) {
     if (n_terms < 0 || n_terms > kExactMaxTerms)
         return fail(SFSEG_ERR_INVALID_ARG, "n_terms must be in [0, 120] (0: chosen from alpha and f's range)");
@@ -690,6 +690,10 @@ int exact_terms(sfseg_handle* h, int n_terms, cudaStream_t s, int* terms_out, fl
     if (!*terms_out)
         return fail(SFSEG_ERR_UNSUPPORTED, "alpha * max(f)^2 too large for the series form of the exact kernel");
     if (h->alpha * (fmax - fmin) * (fmax - fmin) <= kCentredRange) {
+        if (!h->exg && dalloc(&h->exg, (size_t)h->NP) != cudaSuccess) {
+            cudaGetLastError();
+            return SFSEG_OK;
+        }
         *center = (float)(0.5 * (fmax + fmin));
         const double r = std::max(fmax - *center, *center - fmin), x = 2.0 * h->alpha * r * r;
         *terms_out = series_length(x, x);   // products g_i g_j may be negative: sum >= e^-x
@@ -697,19 +701,31 @@ int exact_terms(sfseg_handle* h, int n_terms, cudaStream_t s, int* terms_out, fl
     return SFSEG_OK;
 }
 
-// S = s sum_n c_n g^n G*(g^n w) for w in exv (which it uses up), s = 1/sqrt(*acc) (or 1).
-int exact_series(sfseg_handle* h, const Taps& tp, int terms, const double* acc, float* S, cudaStream_t s) {
+// The exact operator's volumes: w and the term inputs made of it in vbuf[1], the series' sum S in
+// vbuf[0], g (f itself when c = 0) and A.
+struct ExactVolumes {
+    float *v, *S;
+    const float *g, *A;
+};
+ExactVolumes exact_volumes(sfseg_handle* h, float center, cudaStream_t s) {
+    float* gf = center != 0.f ? h->exg : nullptr;
+    launch_exact_setup(h->f32, center, (float)h->alpha, (float)h->p, h->g, gf, h->exa, s);
+    return {(float*)h->vbuf[1], (float*)h->vbuf[0], gf ? gf : h->f32, h->exa};
+}
+
+// S = s sum_n c_n g^n G*(g^n w) for w in e.v (which it uses up), s = 1/sqrt(*acc) (or 1).
+int exact_series(sfseg_handle* h, const ExactVolumes& e, const Taps& tp, int terms, const double* acc, cudaStream_t s) {
     const double a = h->alpha;
     std::vector<double> c((size_t)terms + 2, 0.0);
     c[0] = 1.0;
     for (int n = 1; n < terms; ++n) c[n] = c[n - 1] * 2.0 * a / n;
     const int groups = (terms + 2) / 3;
     for (int j = 0; j < groups; ++j) {
-        if (j > 0) launch_exact_next(h->exg, h->g, h->exv, s);
+        if (j > 0) launch_exact_next(e.g, h->g, e.v, s);
         ExactTerm ex;
         ex.j = j;
         for (int i = 0; i < 3; ++i) ex.c[i] = 3 * j + i < terms ? (float)c[3 * j + i] : 0.f;
-        if (!launch_exact_term_fast(h->exv, S, h->exg, h->g, tp, ex, acc, h->flags, s))
+        if (!launch_exact_term_fast(e.v, e.S, e.g, h->g, tp, ex, acc, h->flags, s))
             return fail(SFSEG_ERR_CUDA, "the TMA stencil could not be launched");
         SFSEG_LAUNCHED();
     }
@@ -721,8 +737,7 @@ int exact_checks(sfseg_handle* h, const Taps& tp) {
     if (h->sep) return fail(SFSEG_ERR_UNSUPPORTED, "the exact kernel is for shared maps (S = F)");
     if (!fast_iterate_supported(tp))
         return fail(SFSEG_ERR_UNSUPPORTED, "the exact kernel runs on the radii with a TMA kernel only");
-    for (float** q : {&h->exv, &h->exg, &h->exa})
-        if (!*q) SFSEG_CUDA(dalloc(q, (size_t)h->NP));
+    if (!h->exa) SFSEG_CUDA(dalloc(&h->exa, (size_t)h->NP));
     return SFSEG_OK;
 }
 }  // namespace
@@ -739,12 +754,11 @@ int sfseg_apply_exact(sfseg_handle* h, const sfseg_neighborhood* nb, int n_terms
     int terms = 0;
     float center = 0.f;
     if (int rc = exact_terms(h, n_terms, s, &terms, &center)) return rc;
-    float* S = (float*)h->vbuf[0];
-    launch_exact_setup(h->f32, center, (float)h->alpha, (float)h->p, h->g, h->exg, h->exa, s);
-    launch_exact_in(x, h->exa, h->g, h->exv, nullptr, s);
+    const ExactVolumes e = exact_volumes(h, center, s);
+    launch_exact_in(x, e.A, h->g, e.v, nullptr, s);
     SFSEG_LAUNCHED();
-    if (int rc = exact_series(h, tp, terms, nullptr, S, s)) return rc;
-    launch_exact_out(S, h->exa, (float)(1.0 / h->alpha), h->g, y, nullptr, s);
+    if (int rc = exact_series(h, e, tp, terms, nullptr, s)) return rc;
+    launch_exact_out(e.S, e.A, (float)(1.0 / h->alpha), h->g, y, nullptr, s);
     SFSEG_LAUNCHED();
     return SFSEG_OK;
 }
@@ -767,19 +781,18 @@ int sfseg_power_iterate_exact(sfseg_handle* h, const sfseg_neighborhood* nb, int
     double* acc = h->acc;
     SFSEG_CUDA(cudaMemsetAsync(acc, 0, sizeof(double) * (iters + 1), s));
     const float inv_alpha = (float)(1.0 / h->alpha);
-    float* S = (float*)h->vbuf[0];
     const float* x_user = init == SFSEG_INIT_USER ? x_inout : nullptr;
     if (iters == 0) {   // x0 itself, normalised
         if (!x_user) launch_fill(x_inout, h->N, 1.f, s);
         launch_sumsq(x_inout, h->N, acc, s);
     } else {
-        launch_exact_setup(h->f32, center, (float)h->alpha, (float)h->p, h->g, h->exg, h->exa, s);
-        launch_exact_in(x_user, h->exa, h->g, h->exv, acc, s);
+        const ExactVolumes e = exact_volumes(h, center, s);
+        launch_exact_in(x_user, e.A, h->g, e.v, acc, s);
         SFSEG_LAUNCHED();
         for (int k = 0; k < iters; ++k) {
-            if (int rc = exact_series(h, tp, terms, acc + k, S, s)) return rc;
-            if (k + 1 < iters) launch_exact_mid(S, h->exa, inv_alpha, h->g, h->exv, acc + k + 1, s);
-            else launch_exact_out(S, h->exa, inv_alpha, h->g, x_inout, acc + iters, s);
+            if (int rc = exact_series(h, e, tp, terms, acc + k, s)) return rc;
+            if (k + 1 < iters) launch_exact_mid(e.S, e.A, inv_alpha, h->g, e.v, acc + k + 1, s);
+            else launch_exact_out(e.S, e.A, inv_alpha, h->g, x_inout, acc + iters, s);
         }
     }
     launch_scale_inv_norm(x_inout, h->N, acc + iters, h->flags, s);

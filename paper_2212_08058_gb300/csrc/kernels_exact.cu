@@ -66,7 +66,7 @@ __global__ void exact_range_kernel(const float* f, Geom g, unsigned* keys) {
 __global__ void exact_setup_kernel(const float* f, float center, float alpha, float p, Geom g, float* gf, float* A) {
     for_each_voxel(g, [&](int64_t, int64_t j) {
         const float fv = f[j], gv = fv - center;
-        gf[j] = gv;
+        if (gf) gf[j] = gv;
         A[j] = unary_pow_fast(fv, p) * expf(-alpha * gv * gv);
     });
 }

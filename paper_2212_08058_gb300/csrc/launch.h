@@ -91,7 +91,7 @@ bool launch_exact_term_fast(const float* v, float* y, const float* gf, const Geo
                             const ExactTerm& ex, const double* acc_in, int* flags, cudaStream_t s);
 
 // The exact kernel's element-wise parts (kernels_exact.cu, internal layout unless noted).  Keys of
-// max f and of max(-f) over the voxels (order_key.cuh; zero both first); g = f - c and
+// max f and of max(-f) over the voxels (order_key.cuh; zero both first); g = f - c (gf nullable) and
 // A = u e^{-alpha g^2}; the first step's w = A x0 (x0 the caller's, or 1) with acc += ||x0||^2; the next
 // step's w = A x~ with x~ = A S / alpha and acc += ||x~||^2; v = g^3 v in place; and the caller's
 // x~ = A S / alpha with acc += ||x~||^2.  acc is nullable.
