@@ -847,19 +847,35 @@ int sfseg_backward(sfseg_handle* h, const sfseg_neighborhood* nb, const float* g
     for (int i = 0; i < 2; ++i)
         if (!h->gbuf[i]) SFSEG_CUDA(dalloc(&h->gbuf[i], (size_t)h->NP));
     if (!h->gz) SFSEG_CUDA(dalloc(&h->gz, (size_t)h->NP));
-    const bool fast_adj = fast_step_supported(tp);
-    if (fast_adj)
-        for (float*& q : h->adjw)
-            if (!q) SFSEG_CUDA(dalloc(&q, (size_t)h->NP));
     while ((int)h->seg.size() < c + 1) {
         float* q = nullptr;
         SFSEG_CUDA(dalloc(&q, (size_t)h->NP));
         h->seg.push_back(q);
     }
-    while (fast_adj && (int)h->qxs.size() < c) {
-        float* q = nullptr;
-        SFSEG_CUDA(dalloc(&q, (size_t)h->NP));
-        h->qxs.push_back(q);
+    bool fast_adj = fast_step_supported(tp);
+    if (fast_adj) {
+        // The state form needs three volumes, and one per step of a segment, that the six-signal form does
+        // not.  Where they do not fit, a radius without its own kernel takes the latter.  Only what this
+        // call allocated is given back: a captured graph may hold the rest.
+        std::vector<float**> fresh;
+        const size_t nq = h->qxs.size();
+        if ((int)nq < c) h->qxs.resize((size_t)c, nullptr);
+        for (float*& q : h->adjw)
+            if (!q) fresh.push_back(&q);
+        for (float*& q : h->qxs)
+            if (!q) fresh.push_back(&q);
+        cudaError_t e = cudaSuccess;
+        for (size_t i = 0; i < fresh.size() && e == cudaSuccess; ++i) e = dalloc(fresh[i], (size_t)h->NP);
+        if (e != cudaSuccess) {
+            for (float** q : fresh) {
+                cudaFree(*q);
+                *q = nullptr;
+            }
+            h->qxs.resize(nq);
+            if (e != cudaErrorMemoryAllocation || fast_iterate_supported(tp)) SFSEG_CUDA(e);
+            cudaGetLastError();
+            fast_adj = false;
+        }
     }
     if (int rc = ensure_acc(&h->dots, &h->dots_cap, K + 2)) return rc;
     // The launch sequence of the reverse pass (capturable: no allocation, no host synchronisation).

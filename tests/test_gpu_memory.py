@@ -65,3 +65,30 @@ def test_exact_operator_in_little_memory(sf, n_terms):
         with _Full((32 + 32 + 24) * MB):     # the output, one volume, and less than another
             y = h.apply_exact(x, r, n_terms=n_terms)
     assert float((y - ref).abs_().max()) <= 2.5e-5 * float(ref.max())
+
+
+def test_reverse_pass_of_a_padded_radius_in_little_memory(sf):
+    """30 steps recorded as one segment, volumes of 8 MB.  With room for the segment's iterates and the
+    three gradient volumes (272 MB), not for the Q of every step that the stencil kernels' form keeps
+    (264 MB more), a radius without a kernel of its own takes the form that needs none.  Same gradient:
+    roundings of 30 steps of float32, 30 * (2 (1 + 6 + 6) + 3 + 12) * 2^-24 = 7.3e-5 of the largest,
+    twice for the pass back."""
+    T, H, W, r = 8, 512, 512, (1, 6, 6)
+    g = torch.Generator(device="cuda").manual_seed(31)
+    V = torch.rand((2, T, H, W), device="cuda", generator=g)
+    c = torch.randn((T, H, W), device="cuda", generator=g)
+    w = [0.8, -0.5]
+    out = []
+    for leave in (None, 272 * MB + 100 * MB):
+        with sf.PowerIteration(2, T, H, W) as h:
+            x = h.power_iterate(V, w, 0.1, r, iters=30, record_every=30)
+            if leave is None:
+                gw, gb = h.backward(c, r)
+            else:
+                with _Full(leave):
+                    gw, gb = h.backward(c, r)
+                    gw2, gb2 = h.backward(c, r)
+                    np.testing.assert_allclose(np.append(gw2, gb2), np.append(gw, gb), rtol=1e-6)
+            del x
+            out.append(np.append(gw, gb).astype(np.float64))
+    assert np.abs(out[0] - out[1]).max() <= 1.5e-4 * np.abs(out[0]).max()
