@@ -157,6 +157,7 @@ struct Params {
     int exj;
     float exc[3];     // c_{3j}, c_{3j+1}, c_{3j+2}
     unsigned* maxkey; // MODE 8: atomicMax of the order key of the largest output
+    bool nan_key;     // MODE 8: a NaN among the outputs makes the key a NaN's
 };
 
 // The tensor maps: halo boxes of v and f; tiles of f, of the second input, and of both outputs.
@@ -209,7 +210,9 @@ __device__ __forceinline__ bool run_of(const Params& P, int s, Run& r) {
 // (writes it when j = 0).  All in the internal layout.  MODE 8 writes x~ in the
 // internal layout and adds the largest of its outputs to P.maxkey (atomicMax of the order key, one per
 // warp; nullable): the maximum a soft-binarisation step (Alg. 1 step 3) scales by, without a pass of its
-// own.  The last step of a power iteration is one too, without the key.
+// own.  fmaxf drops a NaN; for a radius without its own kernel, whose zero taps would spread it further
+// than its neighbourhood, P.nan_key lets it through, as a maximum over the written outputs would (the sum
+// of squares is a NaN exactly when an output was).  The last step of a power iteration is one too, without the key.
 template <int RT, int RH, int RW, typename TS, typename TVO, bool OUT_X, bool SEP, int MODE>
 __global__ void __launch_bounds__(NTHR, 1)
 iter_stream(const __grid_constant__ Maps M, const __grid_constant__ Params P) {
@@ -591,7 +594,8 @@ iter_stream(const __grid_constant__ Maps M, const __grid_constant__ Params P) {
         }
         red[i] += (double)part.x + (double)part.y;
         if constexpr (MODE == 8) {
-            const unsigned kmax = __reduce_max_sync(0xffffffffu, order_key(tmax));
+            const unsigned key = P.nan_key && isnan(red[i]) ? kNanKey : order_key(tmax);
+            const unsigned kmax = __reduce_max_sync(0xffffffffu, key);
             if (lane == 0 && P.maxkey) atomicMax(P.maxkey, kmax);
         }
     }
@@ -641,6 +645,7 @@ static bool launch_t(const StepArgs& a) {
     P.exj = a.ex ? a.ex->j : 0;
     for (int i = 0; i < 3; ++i) P.exc[i] = a.ex ? a.ex->c[i] : 0.f;
     P.maxkey = a.maxkey;
+    P.nan_key = a.tp.rt != RT || a.tp.rh != RH || a.tp.rw != RW;
     P.tx = (g.W + TW - 1) / TW;
     P.tiles = P.tx * ((g.H + TH - 1) / TH);
     const int64_t frames = (int64_t)P.tiles * g.T;   // output frames of all tiles

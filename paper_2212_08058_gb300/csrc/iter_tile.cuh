@@ -94,6 +94,7 @@ struct Params {
     int exj;
     float exc[3];     // c_{3j}, c_{3j+1}, c_{3j+2}
     unsigned* maxkey; // MODE 8: atomicMax of the order key of the largest output
+    bool nan_key;     // MODE 8: a NaN among the outputs makes the key a NaN's
 };
 
 // SEP and MODE as at iter_stream (iter_stream.cuh).
@@ -419,7 +420,8 @@ iter_tile(const __grid_constant__ CUtensorMap mv, const __grid_constant__ CUtens
     if (tid == 0 && P.acc_out) atomicAdd(P.acc_out, tot);
     if constexpr (MODE == 8) {
         __shared__ unsigned wmax[NTHR / 32];
-        const unsigned kmax = __reduce_max_sync(0xffffffffu, order_key(tmax));
+        const unsigned key = P.nan_key && isnan(part.x + part.y) ? kNanKey : order_key(tmax);
+        const unsigned kmax = __reduce_max_sync(0xffffffffu, key);
         if (lane == 0) wmax[warp] = kmax;
         __syncthreads();
         if (tid == 0) {
@@ -467,6 +469,7 @@ static bool launch_t(const StepArgs& a) {
     P.exj = a.ex ? a.ex->j : 0;
     for (int i = 0; i < 3; ++i) P.exc[i] = a.ex ? a.ex->c[i] : 0.f;
     P.maxkey = a.maxkey;
+    P.nan_key = a.tp.rt != RT || a.tp.rh != RH || a.tp.rw != RW;
     const int tx = (g.W + TW - 1) / TW, ty = (g.H + TH - 1) / TH;
     P.tchunk = tile_chunk(g.T, tx * ty, slots_per_sm * num_sms(), RT);
     P.acc_in = a.acc_in;

@@ -10,6 +10,7 @@ __device__ __forceinline__ unsigned order_key(float v) {
     const unsigned b = __float_as_uint(v);
     return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
 }
+constexpr unsigned kNanKey = 0xffffffffu;   // of a NaN: above every number's key
 __device__ __forceinline__ float order_value(unsigned k) {
     return __uint_as_float((k & 0x80000000u) ? (k & 0x7fffffffu) : ~k);
 }

@@ -87,3 +87,24 @@ def test_soft_binarize_errors(sf):
         h.set_features(torch.rand((1, 2, 8, 8), device="cuda") + 0.1)
         xs, m = h.soft_binarize(x, (1, 3, 3), iters=2)
         assert bool(((xs > 0) & (xs < 1)).all())
+
+
+@pytest.mark.parametrize("bad", [float("nan"), float("inf")])
+@pytest.mark.parametrize("T,H,W", [(4, 40, 70), (40, 200, 300)])
+@pytest.mark.parametrize("radius", [(1, 6, 6), (0, 1, 1), (3, 1, 2)])
+def test_non_finite_x_stops_the_step(sf, radius, T, H, W, bad):
+    """A NaN or Inf in the caller's x makes the maximum of A x a NaN for a radius without a kernel of its
+    own, whichever kernel runs it: the call says so, and x stays."""
+    g = torch.Generator(device="cuda").manual_seed(8)
+    V = torch.rand((1, T, H, W), device="cuda", generator=g) + 0.1
+    x = torch.rand((T, H, W), device="cuda", generator=g)
+    x[T // 2, H // 3, W // 2] = bad
+    with sf.PowerIteration(1, T, H, W) as h:
+        h.set_features(V)
+        x0 = x.clone()
+        with pytest.raises(sf.SFSegError) as e:
+            h.soft_binarize(x, radius, iters=3, inplace=True)
+        assert e.value.status == "ZERO_NORM"
+        assert torch.equal(x.view(torch.int32), x0.view(torch.int32))
+        xs, _ = h.soft_binarize(torch.rand((T, H, W), device="cuda", generator=g), radius, iters=2)
+        assert bool(((xs > 0) & (xs < 1)).all())
