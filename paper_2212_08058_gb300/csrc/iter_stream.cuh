@@ -64,6 +64,7 @@ static_assert(kRegsW >= 128 && kRegsH <= 128 && kRegsIO <= 128 && kRegsW % 8 == 
 constexpr int NSTAGE = 3;      // halo boxes in flight
 constexpr int NQ = 2;          // h-pass results in the ring (three: the same time)
 constexpr int NSEG = TW / 8;
+constexpr int kFold = 32;      // frames whose squares are summed in float32
 
 __device__ __forceinline__ void tma_store_3d(const CUtensorMap* map, const void* src, int x, int y, int z) {
     asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.bulk_group [%0, {%1, %2, %3}], [%4];" ::"l"(map), "r"(x),
@@ -424,11 +425,11 @@ iter_stream(const __grid_constant__ Maps M, const __grid_constant__ Params P) {
         // 2rt running partial sums of the 2rt+1-tap filter; with x[n] the w-filtered frame n and
         // g_j = gt[2rt - j], the output y[n] = sum_j g_j x[n - j] is the t-filtered frame n - rt.
         float2 st[2 * RT > 0 ? 2 * RT : 1][3][4];
-        // The norm (or dot product): a run's frames in float32, the runs in FP64 in shared memory.  In
-        // float32 over all of a CTA's runs, volumes of many tiles lost digits: 26 tiles of 20 equal
-        // frames put the norm 1.2e-5 off, against 3e-7 by run.  The fold stands at a run's start: at its
-        // end, or by frame, the compiler's schedule of the passes is worse (144 us; here 138.2, and
-        // 137.7 without it).
+        // The norm (or dot product): kFold output frames in float32, those sums in FP64 in shared memory.
+        // One float32 sum over a long run loses digits: 500 equal frames put the norm 1.2e-5 off, where
+        // 128 squares per sum are at most 3.8e-6 away.  The fold stands with the output frame's inputs, where
+        // it costs nothing (50 steps at 480p 7391 us); around the frame loop they took 7419, at its head 7435,
+        // and a step with the fold at the frame's end 144 us against 138.
         float2 part = make_float2(0.f, 0.f);
         red[i] = 0.0;
         float tmax = 0.f;   // MODE 8: the largest output so far (outputs are >= 0)
@@ -437,8 +438,6 @@ iter_stream(const __grid_constant__ Maps M, const __grid_constant__ Params P) {
         int q = 0, qp = 0, e = 0;           // Q ring slot and phase; output frames finished so far
         Run r;
         for (int s = 0; ok && run_of(P, s, r); ++s) {
-            red[i] += (double)part.x + (double)part.y;
-            part = make_float2(0.f, 0.f);
 #pragma unroll
             for (int a = 0; a < 2 * RT; ++a)
 #pragma unroll
@@ -452,6 +451,10 @@ iter_stream(const __grid_constant__ Maps M, const __grid_constant__ Params P) {
                 const int b = e & 1;
                 float2 fo[4], so[4], uo[4];
                 if (emit) {
+                    if (e % kFold == 0) {
+                        red[i] += (double)part.x + (double)part.y;
+                        part = make_float2(0.f, 0.f);
+                    }
                     const uint32_t ph = (uint32_t)(e >> 1) & 1;
                     ok = mbar_wait_bounded(&ffull[b], ph) && (e < 2 || mbar_wait_bounded(&oempty[b], ph ^ 1));
                     ld_cols(reinterpret_cast<const TS*>(smem + C::O_F + b * C::FT) + tile_off, fo);

@@ -149,3 +149,16 @@ def test_exact_refusals_stay(sf):
         with pytest.raises(sf.SFSegError) as e:
             h.apply_exact(torch.rand((4, 20, 30), device="cuda"), (1, 3, 3))
         assert e.value.status == "UNSUPPORTED"
+
+
+def test_norm_of_many_frames(sf):
+    """The Eq. 8 norm of 500 equal frames of 152 tiles, one run of 500 frames per SM: at most 32 frames
+    go into one float32 sum of 128 equal squares per lane, each addition 2^-24 of the sum away at most,
+    so the root of the sum 128 * 2^-25 = 3.8e-6."""
+    T, H, W, r = 500, 342, 896, (1, 3, 3)
+    with sf.PowerIteration(1, T, H, W) as h:
+        V = torch.full((1, T, H, W), 0.37, device="cuda")
+        _, nu = h.power_iterate(V, radius=r, iters=1, return_norms=True)
+        x0 = torch.full((T, H, W), (T * H * W) ** -0.5, device="cuda")
+        y = h.apply(x0, r)
+    assert abs(float(nu[0]) / float(y.double().norm()) - 1.0) <= 3.8e-6
