@@ -872,27 +872,40 @@ wgrad_tc(const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUten
 // 3 (dh + 1) + (dw + 1) from row block j = dh + 1, dz frame s = 1 - dt; db[co] from the first constant
 // row block of the dz frame s = 1 (the others repeat it).  A block sums 32 values, each of its
 // warps every kRedWarps-th partial: one thread per value walked 152 partials 147 KB apart, 28 us of
-// memory latency for 22 MB.  Sums are kept as hi + lo, the error-free transformation of each addition
-// (Knuth's TwoSum), to about 48 bits like FP64 would, at FP32 rate.
+// memory latency for 22 MB.  Sums are kept as hi + mid + lo, the error-free transformation of each
+// addition (Knuth's TwoSum) twice, at FP32 rate: over 70 bits, where FP64 (2 additions per clock per SM, and
+// as many conversions) has 53.  What leaves float32's range on the way is summed again in FP64.
 constexpr int kRedWarps = 8;
-struct TwoFloat {
-    float hi = 0.f, lo = 0.f;
+struct ThreeFloat {
+    float hi = 0.f, mid = 0.f, lo = 0.f;
+    // s += v; returns what the rounding of that lost
+    static __device__ __forceinline__ float two_sum(float& s, float v) {
+        const float t = __fadd_rn(s, v), z = __fsub_rn(t, s);
+        const float e = __fadd_rn(__fsub_rn(s, __fsub_rn(t, z)), __fsub_rn(v, z));
+        s = t;
+        return e;
+    }
     __device__ __forceinline__ void add(float v) {
-        const float t = __fadd_rn(hi, v), z = __fsub_rn(t, hi);
-        lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(t, z)), __fsub_rn(v, z)));
-        hi = t;
+        const float e = two_sum(hi, v);
+        lo = __fadd_rn(lo, two_sum(mid, e));
+    }
+    __device__ __forceinline__ float value() const {
+        float s = hi;
+        const float e = two_sum(s, mid);
+        return __fadd_rn(s, __fadd_rn(e, lo));
     }
 };
 template <int NCI, int NCO>
 __global__ void __launch_bounds__(32 * kRedWarps)
 wgrad_reduce(const float* part, int nparts, int cout, int cin, float* dW, float* db) {
     using C = WgCfg<NCI, NCO>;
-    __shared__ TwoFloat sums[kRedWarps][32];
+    __shared__ ThreeFloat sums[kRedWarps][32];
     wait_previous_grid();
     const int total = cout * 27 * cin;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int idx = blockIdx.x * 32 + lane;
-    TwoFloat acc;
+    ThreeFloat acc;
+    const float* p0 = part;
     if (idx < total + cout) {
         int n, m, dw;
         if (idx < total) {
@@ -907,7 +920,7 @@ wgrad_reduce(const float* part, int nparts, int cout, int cin, float* dW, float*
             n = NCO * 8 + co;
             m = 3 * C::XC;
         }
-        const float* p0 = part + ((size_t)dw * C::N + n) * 128 + m;
+        p0 = part + ((size_t)dw * C::N + n) * 128 + m;
 #pragma unroll 4
         for (int p = warp; p < nparts; p += kRedWarps) acc.add(p0[(size_t)p * C::PART]);
     }
@@ -916,10 +929,17 @@ wgrad_reduce(const float* part, int nparts, int cout, int cin, float* dW, float*
     if (warp == 0 && idx < total + cout) {
         for (int w = 1; w < kRedWarps; ++w) {
             acc.add(sums[w][lane].hi);
-            acc.lo = __fadd_rn(acc.lo, sums[w][lane].lo);
+            acc.add(sums[w][lane].mid);
+            acc.add(sums[w][lane].lo);
         }
-        if (idx < total) dW[idx] = acc.hi + acc.lo;
-        else db[idx - total] = acc.hi + acc.lo;
+        float r = acc.value();
+        if (!isfinite(r)) {
+            double d = 0.0;
+            for (int p = 0; p < nparts; ++p) d += (double)p0[(size_t)p * C::PART];
+            r = (float)d;
+        }
+        if (idx < total) dW[idx] = r;
+        else db[idx - total] = r;
     }
 }
 

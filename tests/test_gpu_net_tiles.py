@@ -282,3 +282,25 @@ def test_network_sampled_at_production_tile_heights(sf, shape, fr, hr):
     assert np.all(gots > 0)
     assert np.abs(gots - refs).max() <= 3e-2 * np.abs(refs).max(), float(np.abs(gots - refs).max())
     net.close()
+
+
+def test_weight_gradient_sums_of_unlike_size(sf):
+    """db = sum dz over rows that different CTAs sum, as in FP64: Inf stays Inf, a sum whose first parts
+    overflow float32 together comes back with the third, and a small part survives two larger ones that
+    cancel (each value is a bf16 number, each FP64 sum exact)."""
+    T, H, W = 4, 38, 32                      # 152 rows: one per CTA
+    big = 2.0 ** 127
+    net = sf.WarmStartNet(9, seed=1)
+    x = torch.zeros((T, H, W, 32), device="cuda", dtype=torch.bfloat16)
+    dz = torch.zeros((T, H, W, 32), device="cuda", dtype=torch.bfloat16)
+    for h, v in enumerate((big, big, -big)):
+        dz[0, h, 3, 0] = v
+    dz[0, 0, 2:6, 1] = big                   # 2^129 in one row
+    for h, v in enumerate((2.0 ** 50, 2.0 ** 25, 1.5, -(2.0 ** 50), -(2.0 ** 25))):
+        dz[0, 8 * h, 3, 2] = v               # rows that one warp adds
+        dz[1, h, 3, 3] = v                   # and rows of different ones
+    _, dW, db = net.layer_backward(1, x, dz, want_dx=False)
+    net.close()
+    assert float(db[0]) == big and float(db[1]) == float("inf")
+    assert float(db[2]) == 1.5 and float(db[3]) == 1.5
+    assert float(db[4:].abs().max()) == 0.0 and float(dW.abs().max()) == 0.0
