@@ -1161,19 +1161,22 @@ int ensure_ws(sfseg_net* n, int64_t N, bool train) {
         cudaFree(n->dz16); cudaFree(n->dza); cudaFree(n->dzb); cudaFree(n->z4); cudaFree(n->x0);
         n->x16 = n->a1 = n->a2 = n->a3 = n->dz16 = n->dza = n->dzb = nullptr;
         n->z4 = n->x0 = nullptr;
-        n->cap = 0;
-        NET_CUDA(cudaMalloc(&n->x16, N * 16 * 2));
-        NET_CUDA(cudaMalloc(&n->a1, N * 32 * 2));
-        NET_CUDA(cudaMalloc(&n->a2, N * 32 * 2));
         n->cap = N;
     }
-    if (train && !n->dz16) {
-        NET_CUDA(cudaMalloc(&n->z4, n->cap * 4));
-        NET_CUDA(cudaMalloc(&n->x0, n->cap * 4));
-        NET_CUDA(cudaMalloc(&n->a3, n->cap * 32 * 2));
-        NET_CUDA(cudaMalloc(&n->dz16, n->cap * 16 * 2));
-        NET_CUDA(cudaMalloc(&n->dza, n->cap * 32 * 2));
-        NET_CUDA(cudaMalloc(&n->dzb, n->cap * 32 * 2));
+    // each buffer by itself: an allocation that fails leaves those before it to the next call
+    auto need = [&](auto** p, int64_t bytes) { return *p ? cudaSuccess : cudaMalloc(p, n->cap * bytes); };
+    cudaError_t e = need(&n->x16, 16 * 2);
+    if (e == cudaSuccess) e = need(&n->a1, 32 * 2);
+    if (e == cudaSuccess) e = need(&n->a2, 32 * 2);
+    if (e != cudaSuccess) n->cap = 0;   // the next call, of a smaller volume perhaps, starts anew
+    NET_CUDA(e);
+    if (train) {
+        NET_CUDA(need(&n->z4, 4));
+        NET_CUDA(need(&n->x0, 4));
+        NET_CUDA(need(&n->a3, 32 * 2));
+        NET_CUDA(need(&n->dz16, 16 * 2));
+        NET_CUDA(need(&n->dza, 32 * 2));
+        NET_CUDA(need(&n->dzb, 32 * 2));
     }
     return SFSEG_OK;
 }

@@ -92,3 +92,48 @@ def test_reverse_pass_of_a_padded_radius_in_little_memory(sf):
             del x
             out.append(np.append(gw, gb).astype(np.float64))
     assert np.abs(out[0] - out[1]).max() <= 1.5e-4 * np.abs(out[0]).max()
+
+
+@pytest.mark.parametrize("leave", [100 * MB, 240 * MB])
+def test_training_after_an_allocation_failed(sf, leave):
+    """A training call that runs out of memory part of the way (2M voxels: z and x0 of 8 MB each, then
+    128 + 64 + 128 + 128 MB) reports it, holds on to nothing twice when it is called again, and works
+    once there is room, with the gradients of a network that never ran short."""
+    T, H, W = 8, 512, 512
+    g = torch.Generator(device="cuda").manual_seed(33)
+    feats = torch.rand((3, T, H, W), device="cuda", generator=g).to(torch.bfloat16)
+    target = torch.rand((T, H, W), device="cuda", generator=g)
+    ref = sf.WarmStartNet(3, seed=5)
+    loss0, g0 = ref.backward(feats, target, want_grads=True)
+    ref.close()
+    net = sf.WarmStartNet(3, seed=5)
+    net.forward(feats)
+    with _Full(leave):
+        free = []
+        for _ in range(3):
+            with pytest.raises(sf.SFSegError) as e:
+                net.backward(feats, target)
+            assert e.value.status == "OOM"
+            free.append(torch.cuda.mem_get_info()[0])
+        assert free[0] == free[1] == free[2]
+    loss1, g1 = net.backward(feats, target, want_grads=True)
+    net.close()
+    assert abs(loss1 - loss0) <= 1e-6 and np.array_equal(g0, g1)
+
+
+def test_network_on_a_smaller_volume_after_an_allocation_failed(sf):
+    """A forward pass that does not fit reports it, and a smaller one still works."""
+    g = torch.Generator(device="cuda").manual_seed(34)
+    small = torch.rand((3, 4, 64, 64), device="cuda", generator=g)
+    large = torch.rand((3, 8, 512, 512), device="cuda", generator=g)
+    net = sf.WarmStartNet(3, seed=5)
+    with _Full(200 * MB):                    # 64 + 128 + 128 MB of activations and the result's 8
+        with pytest.raises(sf.SFSegError) as e:
+            net.forward(large)
+        assert e.value.status == "OOM"
+        x0 = net.forward(small).clone()
+    ref = sf.WarmStartNet(3, seed=5)
+    assert torch.equal(x0, ref.forward(small))
+    assert bool(torch.isfinite(net.forward(large)).all())
+    net.close()
+    ref.close()
