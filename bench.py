@@ -895,7 +895,7 @@ def main():
         step(feats, x)
     torch.cuda.synchronize()
     n_launch0 = sfseg.kernel_launches()
-    tma0, gen0, _ = sfseg.iterate_kernel_stats()
+    ran0 = sfseg.step_kernels()
 
     # ---- device-resident timed region
     h.enable_iter_timing(True)
@@ -912,10 +912,12 @@ def main():
         torch.cuda.synchronize()
     ms = ev0.elapsed_time(ev1)
     launches = sfseg.kernel_launches() - n_launch0
-    tma1, gen1, kernel_name = sfseg.iterate_kernel_stats()
-    if gen1 != gen0 or tma1 - tma0 != args.steps * ITERS:
-        raise RuntimeError(f"the timed steps did not all run on the TMA kernel: {tma1 - tma0} TMA steps, "
-                           f"{gen1 - gen0} generic-stencil steps for {args.steps * ITERS} iterations")
+    ran1 = sfseg.step_kernels()
+    on_stream, on_tile, on_stencil = (b - a for a, b in zip(ran0[:3], ran1[:3]))
+    kernel_name = ran1[3]
+    if on_stencil or on_stream + on_tile != args.steps * ITERS:
+        raise RuntimeError(f"the timed steps did not all run on the TMA kernels: {on_stream} + {on_tile} there, "
+                           f"{on_stencil} on the generic stencil, for {args.steps * ITERS} iterations")
     clk_summary = clk.summary()
     it_ms, it_n = h.iter_timing()
     h.enable_iter_timing(False)
@@ -1009,8 +1011,8 @@ def main():
                               "step's upload and this step's download overlap the computation)",
                     "last_download_checked": e2e_ok},
             "gpu_launches": launches,
-            "kernel_ran": {"iteration_kernel": kernel_name, "tma_steps": tma1 - tma0,
-                           "generic_stencil_steps": gen1 - gen0},
+            "kernel_ran": {"iteration_kernel": kernel_name, "iter_stream_steps": on_stream,
+                           "iter_tile_steps": on_tile, "generic_stencil_steps": on_stencil},
             "clocks": clk_summary,
             "residual": res, "rho": rho,
             "paper_context": "0.01 s per iteration per 480x854 frame on a GTX Titan X (Maxwell), "

@@ -390,16 +390,26 @@ int sfseg_normalize(sfseg_handle* h, float* x, int64_t n, const double* acc_dev,
  * TIMEOUT, NONFINITE (bad features or a non-finite norm), ZERO_NORM; OK if none is set. */
 int sfseg_check(sfseg_handle* h, void* stream);
 
-/* Which kernel ran the power-iteration steps (instrumentation; no counterpart in the paper).
- * The radii (1,3,3), (2,7,7), (1,4,4), (1,2,2), (1,5,5), (2,3,3), (2,5,5) and (1,7,7) run on the
- * TMA-staged stencil kernel; other
- * radii, or a volume whose tensor maps the driver does not encode, run on the generic streaming
- * stencil, which gives the same results more slowly.  Process-wide counts of steps issued on
- * each (host outputs; steps captured into a CUDA graph count once, at capture), and in
- * last_kernel (host buffer of len >= 1 chars, or NULL) the kernel name of the last step,
- * e.g. "iter_fast<2,7,7,float,float>".  Errors: INVALID_ARG (null count). */
+/* The power-iteration steps by their radius (instrumentation; no counterpart in the paper):
+ * tma_steps counts those of the radii with a kernel of their own, (1,3,3), (2,7,7), (1,4,4), (1,2,2),
+ * (1,5,5), (2,3,3), (2,5,5) and (1,7,7), generic_steps those of all others and of a volume whose tensor
+ * maps the driver does not encode.  What they ran on is sfseg_step_kernels's to say: a radius with
+ * rt <= 2 and none of its own runs on a wider radius's kernel with zero taps.  Process-wide (host
+ * outputs; steps captured into a CUDA graph count once, at capture).  last_kernel (host buffer of
+ * len >= 1 chars, or NULL): "iter_fast: " or "stream_stencil: " for the two kinds of radius, and the
+ * name that sfseg_step_kernels gives.  Errors: INVALID_ARG (null count). */
 int sfseg_iterate_kernel_stats(int64_t* tma_steps, int64_t* generic_steps, char* last_kernel,
                                int len);
+
+/* Which kernels ran the power-iteration steps, process-wide as above: the streaming stencil
+ * iter_stream, the small-volume stencil iter_tile (both TMA-staged, radii with rt <= 2), or the generic
+ * stencil stream_stencil (rt = 3, 4; separate maps in bf16), and in last_kernel the last step's, with
+ * the radius it is compiled for, the types it read and wrote ("x~": the last step's iterate in the
+ * internal layout, "caller x": in the caller's) and, if another, the radius asked for, e.g.
+ * "iter_stream<2,7,7,float,float>" or "iter_tile<1,4,4,float,x~> for radius 1,1,1".
+ * Errors: INVALID_ARG (null count). */
+int sfseg_step_kernels(int64_t* stream_steps, int64_t* tile_steps, int64_t* stencil_steps,
+                       char* last_kernel, int len);
 
 /* No-allocation power iteration (the paper has no counterpart: this is a deployment aid).
  *

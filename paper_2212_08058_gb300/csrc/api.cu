@@ -616,6 +616,17 @@ int sfseg_iterate_kernel_stats(int64_t* tma_steps, int64_t* generic_steps, char*
     return SFSEG_OK;
 }
 
+int sfseg_step_kernels(int64_t* stream_steps, int64_t* tile_steps, int64_t* stencil_steps, char* last_kernel, int len) {
+    if (!stream_steps || !tile_steps || !stencil_steps) return fail(SFSEG_ERR_INVALID_ARG, "null argument");
+    if (last_kernel && len < 1) return fail(SFSEG_ERR_INVALID_ARG, "len must be >= 1");
+    int64_t n[3];
+    step_kernels(n, last_kernel, len);
+    *stream_steps = n[0];
+    *tile_steps = n[1];
+    *stencil_steps = n[2];
+    return SFSEG_OK;
+}
+
 int sfseg_apply(sfseg_handle* h, const sfseg_neighborhood* nb, const float* x, float* y, void* stream) {
     if (int rc = check_handle(h)) return rc;
     Taps tp;

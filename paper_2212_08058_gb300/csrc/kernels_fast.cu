@@ -101,9 +101,15 @@ bool stream_pays(const Geom& g, const Radius& r) {
     return stream <= tile;
 }
 
+thread_local StepKernel g_ran = {};
+
 bool run(const StepArgs& a) {
     const Radius* r = covering_radius(a.tp);
-    return r && (stream_pays(a.g, *r) ? r->stream(a) : r->tile(a));
+    if (!r) return false;
+    const bool stream = stream_pays(a.g, *r);
+    if (!(stream ? r->stream(a) : r->tile(a))) return false;
+    g_ran = {stream, r->rt, r->rh, r->rw};
+    return true;
 }
 
 StepArgs args(int mode, const void* vin, void* out, const void* f, const Geom& g, const Taps& tp, float inv_alpha,
@@ -125,6 +131,8 @@ StepArgs args(int mode, const void* vin, void* out, const void* f, const Geom& g
 }
 
 }  // namespace
+
+StepKernel last_step_kernel() { return g_ran; }
 
 bool fast_iterate_supported(const Taps& tp) { return own_radius(tp) != nullptr; }
 bool fast_step_supported(const Taps& tp) { return covering_radius(tp) != nullptr; }

@@ -103,30 +103,43 @@ struct OpApply {
 };
 
 static std::atomic<int64_t> g_launches{0};
-// Which kernel ran the power-iteration steps: counts of steps issued on the TMA kernel and on the
-// generic stencil, and the name of the last step's kernel instantiation.
-static std::atomic<int64_t> g_steps_tma{0}, g_steps_generic{0};
+// The power-iteration steps so far, by radius (one with a kernel of its own, or not) and by the kernel
+// that ran them (iter_stream, iter_tile, stream_stencil), and the name of the last step's kernel.
+static std::atomic<int64_t> g_steps_own{0}, g_steps_other{0}, g_steps_by[3];
 static std::mutex g_step_mu;
+static bool g_step_own = false;
 static char g_step_name[96] = "";
 
-// `tma`: the step ran on the TMA kernels.  Steps of a radius without its own kernel count as generic
-// ones, whether they ran on a TMA kernel of a wider radius with zero taps or on stream_stencil.
-static void note_step(bool tma, const Taps& tp, int vin_type, int out_type, bool out_x, bool record, bool sep) {
-    const bool own = tma && fast_iterate_supported(tp);
-    (own ? g_steps_tma : g_steps_generic).fetch_add(1, std::memory_order_relaxed);
+// `tma`: the step ran on one of the TMA kernels; `x_out`: what it wrote, for a last step.
+static void note_step(bool tma, const Taps& tp, int vin_type, int out_type, const char* x_out, bool record, bool sep) {
+    const bool own = fast_iterate_supported(tp) && tma;
+    const StepKernel k = tma ? last_step_kernel() : StepKernel{false, tp.rt, tp.rh, tp.rw};
+    (own ? g_steps_own : g_steps_other).fetch_add(1, std::memory_order_relaxed);
+    g_steps_by[tma ? (k.stream ? 0 : 1) : 2].fetch_add(1, std::memory_order_relaxed);
     char buf[96];
-    std::snprintf(buf, sizeof(buf), "%s<%d,%d,%d,%s,%s%s%s>",
-                  own ? "iter_fast" : (tma ? "stream_stencil(padded taps)" : "stream_stencil<OpIter>"), tp.rt, tp.rh,
-                  tp.rw, vin_type == kF32 ? "float" : "bf16",
-                  out_x ? "float(caller x)" : (out_type == kBF16 ? "bf16" : "float"), record ? ",record" : "",
-                  sep ? ",separate maps" : "");
+    const int n = std::snprintf(buf, sizeof(buf), "%s<%d,%d,%d,%s,%s%s%s>",
+                                tma ? (k.stream ? "iter_stream" : "iter_tile") : "stream_stencil", k.rt, k.rh, k.rw,
+                                vin_type == kF32 ? "float" : "bf16",
+                                x_out ? x_out : (out_type == kBF16 ? "bf16" : "float"), record ? ",record" : "",
+                                sep ? ",separate maps" : "");
+    if (k.rt != tp.rt || k.rh != tp.rh || k.rw != tp.rw)
+        std::snprintf(buf + n, sizeof(buf) - n, " for radius %d,%d,%d", tp.rt, tp.rh, tp.rw);
     std::lock_guard<std::mutex> lk(g_step_mu);
     std::memcpy(g_step_name, buf, sizeof(buf));
+    g_step_own = own;
 }
 
 void iterate_kernel_stats(int64_t* tma_steps, int64_t* generic_steps, char* name, int len) {
-    if (tma_steps) *tma_steps = g_steps_tma.load(std::memory_order_relaxed);
-    if (generic_steps) *generic_steps = g_steps_generic.load(std::memory_order_relaxed);
+    *tma_steps = g_steps_own.load(std::memory_order_relaxed);
+    *generic_steps = g_steps_other.load(std::memory_order_relaxed);
+    if (name && len > 0) {
+        std::lock_guard<std::mutex> lk(g_step_mu);
+        const char* by = !g_step_name[0] ? "" : (g_step_own ? "iter_fast: " : "stream_stencil: ");
+        std::snprintf(name, (size_t)len, "%s%s", by, g_step_name);
+    }
+}
+void step_kernels(int64_t counts[3], char* name, int len) {
+    for (int i = 0; i < 3; ++i) counts[i] = g_steps_by[i].load(std::memory_order_relaxed);
     if (name && len > 0) {
         std::lock_guard<std::mutex> lk(g_step_mu);
         std::snprintf(name, (size_t)len, "%s", g_step_name);
@@ -169,29 +182,30 @@ bool launch_iterate(const void* vin, int vin_type, void* out, int out_type, bool
                     const double* acc_in, double* acc_out, int* flags, cudaStream_t s, const float* s32,
                     float* last_xt) {
     using bf = __nv_bfloat16;
+    const char* caller_x = out_x ? "caller x" : nullptr;
     // The last step into the internal layout; a recording one's record is that same volume.
     if (out_x && last_xt && vin_type == kF32 && s32 == nullptr && fast_step_supported(tp) &&
         launch_iterate_fast_last((const float*)vin, last_xt, (const float*)f, g, tp, inv_alpha, p, acc_in, acc_out,
                                  flags, s)) {
-        note_step(true, tp, vin_type, out_type, out_x, ckpt != nullptr, false);
+        note_step(true, tp, vin_type, out_type, "x~", ckpt != nullptr, false);
         return true;
     }
     // The TMA kernel serves the method's radii, recording steps (float32, shared maps) included.
     if (ckpt == nullptr && fast_step_supported(tp) &&
         launch_iterate_fast(vin, vin_type, out, out_type, out_x, f, g, tp, inv_alpha, p, acc_in, acc_out, flags, s,
                             s32)) {
-        note_step(true, tp, vin_type, out_type, out_x, false, s32 != nullptr);
+        note_step(true, tp, vin_type, out_type, caller_x, false, s32 != nullptr);
         return false;
     }
     if (ckpt != nullptr && vin_type == kF32 && s32 == nullptr && fast_step_supported(tp) &&
         launch_iterate_fast_ckpt((const float*)vin, out, out_x, (const float*)f, g, tp, inv_alpha, p, acc_in, acc_out,
                                  ckpt, flags, s)) {
-        note_step(true, tp, vin_type, out_type, out_x, true, false);
+        note_step(true, tp, vin_type, out_type, caller_x, true, false);
         return false;
     }
     // Radii without a TMA kernel, or a tensor map the driver would not encode: the generic
     // streaming stencil (same results, slower); counted so that callers can tell.
-    note_step(false, tp, vin_type, out_type, out_x, ckpt != nullptr, s32 != nullptr);
+    note_step(false, tp, vin_type, out_type, caller_x, ckpt != nullptr, s32 != nullptr);
 #define SFSEG_IT(TVI, TVO, TF, OX) \
     iterate_t<TVI, TVO, TF, OX>(vin, out, f, ckpt, g, tp, inv_alpha, p, acc_in, acc_out, flags, s, s32)
     // A step of the bf16 phase reads v and f in bf16 and writes bf16, or float32 when the next

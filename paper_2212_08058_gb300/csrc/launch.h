@@ -45,6 +45,13 @@ bool launch_iterate(const void* vin, int vin_type, void* out, int out_type, bool
 bool fast_iterate_supported(const Taps& tp);
 // The same, or a wider radius's kernel can run tp padded with zero taps.
 bool fast_step_supported(const Taps& tp);
+// What the calling thread's most recent step on the TMA kernels ran on: the streaming kernel or the
+// small-volume one, compiled for radius (rt, rh, rw).
+struct StepKernel {
+    bool stream;
+    int rt, rh, rw;
+};
+StepKernel last_step_kernel();
 bool launch_iterate_fast(const void* vin, int vin_type, void* out, int out_type, bool out_x, const void* f,
                          const Geom& g, const Taps& tp, float inv_alpha, float p, const double* acc_in,
                          double* acc_out, int* flags, cudaStream_t s, const float* s32 = nullptr);
@@ -215,9 +222,11 @@ int make_taps(const sfseg_neighborhood* nb, Taps* tp);
 // Records `msg` as the thread's sfseg_last_error() text and returns `code`.
 int set_last_error(int code, const char* msg);
 
-// Process-wide counts of power-iteration steps issued on the TMA kernel and on the generic
-// stencil, and the kernel name of the last one (sfseg_iterate_kernel_stats).
+// Process-wide counts of power-iteration steps by their radius (sfseg_iterate_kernel_stats) and by the
+// kernel that ran them (sfseg_step_kernels: iter_stream, iter_tile, stream_stencil), with the last step's
+// name.
 void iterate_kernel_stats(int64_t* tma_steps, int64_t* generic_steps, char* name, int len);
+void step_kernels(int64_t counts[3], char* name, int len);
 
 // Process-wide count of kernels launched by the library (sfseg_kernel_launches).
 void count_launches(int n);

@@ -78,6 +78,8 @@ SIGNATURES = {
     "sfseg_check": [_vp, _vp],
     "sfseg_iterate_kernel_stats": [ctypes.POINTER(ctypes.c_int64), ctypes.POINTER(ctypes.c_int64),
                                    ctypes.c_char_p, _i],
+    "sfseg_step_kernels": [ctypes.POINTER(ctypes.c_int64), ctypes.POINTER(ctypes.c_int64),
+                           ctypes.POINTER(ctypes.c_int64), ctypes.c_char_p, _i],
     "sfseg_net_create": [_i, ctypes.c_uint64, ctypes.POINTER(_vp)],
     "sfseg_net_destroy": [_vp],
     "sfseg_net_num_params": [_vp, ctypes.POINTER(ctypes.c_int64)],
@@ -541,12 +543,21 @@ def net_launch_shape(kernel: int):
 
 
 def iterate_kernel_stats():
-    """(steps on the TMA kernel, steps on the generic stencil, name of the last step's kernel),
-    process-wide."""
+    """(steps of the radii with a kernel of their own, steps of other radii, label and name of the
+    last step's kernel), process-wide; step_kernels() says what ran them."""
     a, b = ctypes.c_int64(), ctypes.c_int64()
     buf = ctypes.create_string_buffer(128)
     _check(lib().sfseg_iterate_kernel_stats(ctypes.byref(a), ctypes.byref(b), buf, len(buf)))
     return a.value, b.value, buf.value.decode()
+
+
+def step_kernels():
+    """(steps on iter_stream, on iter_tile, on the generic stream_stencil, name of the last step's
+    kernel), process-wide (sfseg_step_kernels)."""
+    n = [ctypes.c_int64() for _ in range(3)]
+    buf = ctypes.create_string_buffer(128)
+    _check(lib().sfseg_step_kernels(*(ctypes.byref(v) for v in n), buf, len(buf)))
+    return n[0].value, n[1].value, n[2].value, buf.value.decode()
 
 
 class SFSegFunction(torch.autograd.Function):

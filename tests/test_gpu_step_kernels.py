@@ -162,3 +162,32 @@ def test_norm_of_many_frames(sf):
         x0 = torch.full((T, H, W), (T * H * W) ** -0.5, device="cuda")
         y = h.apply(x0, r)
     assert abs(float(nu[0]) / float(y.double().norm()) - 1.0) <= 3.8e-6
+
+
+@pytest.mark.parametrize("T,H,W,radius,maps,bf16,kernel", [
+    (24, 325, 449, (2, 7, 7), 1, 0, "iter_stream<2,7,7,float,x~>"),
+    (24, 325, 449, (1, 6, 6), 1, 0, "iter_stream<1,7,7,float,x~> for radius 1,6,6"),
+    (24, 325, 449, (1, 3, 3), 2, 0, "iter_stream<1,3,3,float,caller x,separate maps>"),
+    (24, 325, 449, (1, 3, 3), 1, 2, "iter_stream<1,3,3,bf16,caller x>"),
+    (5, 40, 70, (2, 7, 7), 1, 0, "iter_tile<2,7,7,float,x~>"),
+    (5, 40, 70, (0, 1, 1), 1, 0, "iter_tile<1,2,2,float,x~> for radius 0,1,1"),
+    (5, 40, 70, (1, 6, 6), 2, 0, "iter_tile<1,7,7,float,caller x,separate maps> for radius 1,6,6"),
+    (5, 40, 70, (3, 5, 5), 1, 0, "stream_stencil<3,5,5,float,caller x>"),
+    (5, 40, 70, (1, 3, 3), 2, 2, "stream_stencil<1,3,3,bf16,caller x,separate maps>"),
+])
+def test_step_kernels_says_what_ran(sf, T, H, W, radius, maps, bf16, kernel):
+    g = torch.Generator(device="cuda").manual_seed(2)
+    V = torch.rand((1, T, H, W), device="cuda", generator=g)
+    with sf.PowerIteration(1, T, H, W) as h:
+        if maps == 2:
+            h.set_features_sf(V, None, 0.0, V.flip(1).contiguous())
+        else:
+            h.set_features(V)
+        n0 = sf.step_kernels()
+        h.power_iterate(None, radius=radius, iters=2, iters_bf16=bf16)
+        n1 = sf.step_kernels()
+    at = ("iter_stream", "iter_tile", "stream_stencil").index(kernel.split("<")[0])
+    assert [b - a for a, b in zip(n0[:3], n1[:3])] == [2 * (i == at) for i in range(3)]
+    assert n1[3] == kernel
+    label = sf.iterate_kernel_stats()[2]
+    assert label in ("iter_fast: " + kernel, "stream_stencil: " + kernel)
