@@ -46,14 +46,19 @@ __device__ __forceinline__ float unary_pow(float s, float p) {
 
 // Faster variant on the special-function unit: u = 2^(p log2 s) with the approximate log2 and
 // exp2 instructions (relative error a few 1e-7 for p <= 1).  s = 0 gives log2 s = -inf and
-// u = +0, so no branch is needed (s < 0 never reaches here: features are checked >= 0).  lg2 takes
-// subnormal s (its u is not small); u itself below 2^-126 becomes 0 (three instructions less).
+// u = +0, so no branch is needed (s < 0 never reaches here: features are checked >= 0).  Both
+// take and give subnormal numbers; with FTZ a u below 2^-126 becomes 0, three instructions less.
+template <bool FTZ = false>
 __device__ __forceinline__ float unary_pow_fast(float s, float p) {
     float l, u;
     asm("lg2.approx.f32 %0, %1;" : "=f"(l) : "f"(s));
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(u) : "f"(p * l));
+    if constexpr (FTZ) asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(u) : "f"(p * l));
+    else asm("ex2.approx.f32 %0, %1;" : "=f"(u) : "f"(p * l));
     return u;
 }
+// No positive float32 s is below 2^-149, so u is subnormal only for p > 126 / 149 = 0.845: up to this p the
+// shorter form gives the same numbers.
+constexpr float kUnaryFtzP = 0.84f;
 
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll

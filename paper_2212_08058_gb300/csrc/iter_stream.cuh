@@ -463,7 +463,16 @@ iter_stream(const __grid_constant__ Maps M, const __grid_constant__ Params P) {
 #pragma unroll
                     for (int m = 0; m < 4; ++m) {
                         const float2 sv = SEP ? so[m] : fo[m];
-                        uo[m] = make_float2(unary_pow_fast(sv.x, P.p), unary_pow_fast(sv.y, P.p));
+                        uo[m] = make_float2(unary_pow_fast<true>(sv.x, P.p), unary_pow_fast<true>(sv.y, P.p));
+                    }
+                    // again for the rest, in a branch never taken for the usual p: the longer form
+                    // throughout costs 1.4 % (solve 480p 7391 -> 7495 us)
+                    if (P.p > kUnaryFtzP) {
+#pragma unroll
+                        for (int m = 0; m < 4; ++m) {
+                            const float2 sv = SEP ? so[m] : fo[m];
+                            uo[m] = make_float2(unary_pow_fast(sv.x, P.p), unary_pow_fast(sv.y, P.p));
+                        }
                     }
                 }
                 ok = ok && mbar_wait_bounded(&qfull[q], qp);

@@ -297,7 +297,7 @@ iter_tile(const __grid_constant__ CUtensorMap mv, const __grid_constant__ CUtens
             for (int m = 0; m < 4; ++m) {
                 const float2 fv = fo[m];
                 const float2 sv = SEP ? so[SEP ? m : 0] : fv;
-                const float2 u = make_float2(unary_pow_fast(sv.x, P.p), unary_pow_fast(sv.y, P.p));
+                const float2 u = make_float2(unary_pow_fast<true>(sv.x, P.p), unary_pow_fast<true>(sv.y, P.p));
                 const float2 e = fma2(make_float2(-fv.x, -fv.y), fv, f2(P.inv_alpha));   // 1/alpha - f^2
                 if constexpr (MODE == 7) {
                     float2 F = make_float2(1.f, 1.f);

@@ -191,3 +191,26 @@ def test_step_kernels_says_what_ran(sf, T, H, W, radius, maps, bf16, kernel):
     assert n1[3] == kernel
     label = sf.iterate_kernel_stats()[2]
     assert label in ("iter_fast: " + kernel, "stream_stencil: " + kernel)
+
+
+@pytest.mark.parametrize("radius", [(1, 3, 3), (2, 7, 7), (1, 6, 6), (3, 1, 2)])
+@pytest.mark.parametrize("T,H,W", [(1, 1, 2), (4, 30, 40), (3, 37, 230), (40, 325, 561)])
+def test_unary_below_the_normal_range(sf, radius, T, H, W):
+    """u = s^9.6 is 10^-38.4 = 4e-39, a subnormal float32, where s = 1e-4, and 1 elsewhere; the outputs
+    there are ordinary numbers again for x = 1e6.  u's relative error: the product p log2 s = 128 and the
+    logarithm are rounded to 2^-22, so 128 * 2^-21 * ln 2 = 4.2e-5, the rest far below."""
+    f = np.ones((T, H, W), np.float32)
+    at = (T // 2, H // 2, W // 2)
+    f[at] = 1e-4
+    x = np.full((T, H, W), 1e6, np.float32)
+    with sf.PowerIteration(1, T, H, W, p=9.6) as h:
+        h.set_features(torch.from_numpy(f[None]).cuda())
+        y = h.apply(torch.from_numpy(x).cuda(), radius).cpu().numpy()
+        xi, nu = h.power_iterate(None, radius=radius, iters=3, return_norms=True)
+        xi = xi.cpu().numpy()
+    f64 = f.astype(np.float64)
+    yo = oracle.filter_apply(f64, f64, 9.6, 1.0, radius, x.astype(np.float64))
+    assert np.abs(y / yo - 1.0).max() <= 5e-5
+    xo, nuo = oracle.power_filter(f64, f64, 9.6, 1.0, radius, np.ones(f.shape), 3)
+    assert np.abs(xi - xo).max() <= 3 * (2 * sum(radius) + 3 + 12) * 2.0 ** -24 * xo.max()
+    np.testing.assert_allclose(nu, nuo, rtol=1e-5)
