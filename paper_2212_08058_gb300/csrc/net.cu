@@ -930,7 +930,7 @@ wgrad_reduce(const float* part, int nparts, int cout, int cin, float* dW, float*
         for (int w = 1; w < kRedWarps; ++w) {
             acc.add(sums[w][lane].hi);
             acc.add(sums[w][lane].mid);
-            acc.add(sums[w][lane].lo);
+            acc.lo = __fadd_rn(acc.lo, sums[w][lane].lo);
         }
         float r = acc.value();
         if (!isfinite(r)) {
