@@ -230,16 +230,27 @@ static int ensure_acc(double** buf, int* cap, int need) {
     return SFSEG_OK;
 }
 
-static int read_flags(sfseg_handle* h, cudaStream_t s) {
-    int fl = 0;
-    SFSEG_CUDA(cudaMemcpyAsync(&fl, h->flags, sizeof(int), cudaMemcpyDeviceToHost, s));
+// The handle's error flags (synchronises); cleared on the device if any is set.
+static int take_flags(sfseg_handle* h, cudaStream_t s, int* fl) {
+    *fl = 0;
+    SFSEG_CUDA(cudaMemcpyAsync(fl, h->flags, sizeof(int), cudaMemcpyDeviceToHost, s));
     SFSEG_CUDA(cudaStreamSynchronize(s));
-    if (fl) SFSEG_CUDA(cudaMemsetAsync(h->flags, 0, sizeof(int), s));
+    if (*fl) SFSEG_CUDA(cudaMemsetAsync(h->flags, 0, sizeof(int), s));
+    return SFSEG_OK;
+}
+
+static int report_flags(int fl) {
     if (fl & kFlagTimeout) return fail(SFSEG_ERR_TIMEOUT, "a bounded wait for a TMA copy gave up");
     if (fl & kFlagBadFeature) return fail(SFSEG_ERR_NONFINITE, "features must be finite and >= 0");
     if (fl & kFlagNonfinite) return fail(SFSEG_ERR_NONFINITE, "an iterate norm became NaN or Inf");
     if (fl & kFlagZeroNorm) return fail(SFSEG_ERR_ZERO_NORM, "an iterate became zero (u = 0 on its support?)");
     return SFSEG_OK;
+}
+
+static int read_flags(sfseg_handle* h, cudaStream_t s) {
+    int fl = 0;
+    if (int rc = take_flags(h, s, &fl)) return rc;
+    return report_flags(fl);
 }
 
 namespace sfseg {
@@ -1144,13 +1155,16 @@ int sfseg_soft_binarize(sfseg_handle* h, const sfseg_neighborhood* nb, int iters
     };
     if (int rc = steps(false)) return rc;
     int fl = 0;
-    SFSEG_CUDA(cudaMemcpyAsync(&fl, h->flags, sizeof(int), cudaMemcpyDeviceToHost, s));
-    SFSEG_CUDA(cudaStreamSynchronize(s));
+    if (int rc = take_flags(h, s, &fl)) return rc;
     // A step stopped (so did those after it, and x is still the caller's): once more, with x stored by
     // every step, so that x is left as the step before the stop made it.
-    if ((fl & kFlagTailStop) && fast && iters > 1)
+    if ((fl & kFlagTailStop) && fast && iters > 1) {
         if (int rc = steps(true)) return rc;
-    return read_flags(h, s);
+        int again = 0;
+        if (int rc = take_flags(h, s, &again)) return rc;
+        fl |= again;
+    }
+    return report_flags(fl);
 }
 
 int sfseg_selftest_wait(sfseg_handle* h, long long spins, void* stream) {

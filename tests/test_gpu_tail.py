@@ -108,3 +108,27 @@ def test_non_finite_x_stops_the_step(sf, radius, T, H, W, bad):
         assert torch.equal(x.view(torch.int32), x0.view(torch.int32))
         xs, _ = h.soft_binarize(torch.rand((T, H, W), device="cuda", generator=g), radius, iters=2)
         assert bool(((xs > 0) & (xs < 1)).all())
+
+
+@pytest.mark.parametrize("separate", [False, True])
+@pytest.mark.parametrize("radius", [(1, 3, 3), (1, 6, 6), (3, 1, 2)])
+@pytest.mark.parametrize("T,H,W", [(3, 17, 40), (40, 200, 300)])
+def test_stop_at_a_later_step_keeps_the_step_before(sf, T, H, W, radius, separate):
+    """With centre 2 and gain 200 the sigmoid is at most e^-200 = 0 in float32, so A x of the second
+    step is 0 and that step stops: x is what the first step left, as a call of one step gives it."""
+    g = torch.Generator(device="cuda").manual_seed(9)
+    V = torch.rand((2, T, H, W), device="cuda", generator=g)
+    x = torch.rand((T, H, W), device="cuda", generator=g)
+    w = [0.7, 0.4]
+    with sf.PowerIteration(2, T, H, W) as h:
+        if separate:
+            h.set_features_sf(V, w, 0.1, V, w, 0.0)
+        else:
+            h.set_features(V, w, 0.0)
+        one, _ = h.soft_binarize(x, radius, iters=1, gain=200.0, center=2.0)
+        assert float(one.max()) == 0.0
+        y = x.clone()
+        with pytest.raises(sf.SFSegError) as e:
+            h.soft_binarize(y, radius, iters=4, gain=200.0, center=2.0, inplace=True)
+        assert e.value.status == "ZERO_NORM"
+        assert torch.equal(y, one)
