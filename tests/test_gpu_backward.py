@@ -197,3 +197,43 @@ def test_adjoint_graph_replay_is_identical():
     for (a, ab), (b, bb) in zip(outs[False], outs[True]):
         np.testing.assert_allclose(a, b, rtol=1e-6, atol=1e-9 * np.abs(a).max())
         assert abs(ab - bb) <= 1e-6 * max(abs(ab), np.abs(a).max())
+
+
+@pytest.mark.parametrize("K,every,r", [(6, 2, (3, 1, 2)), (5, 5, (3, 1, 2)), (4, 3, (4, 3, 2)), (1, 1, (4, 1, 1))])
+def test_six_signal_adjoint_matches_oracle_gradient(K, every, r):
+    """Radii with rt = 3 and 4, whose reverse pass is the six-signal stencil: the oracle's reverse pass on
+    the explicit matrix, to the bound of the state form's test above (test_adjoint_matches_oracle_gradient)."""
+    V, _, _ = synth.multichannel(6, 12, 12, C=2, seed=4001)
+    w = np.array([1.4, -0.7], dtype=np.float32)
+    rng = np.random.default_rng(11)
+    c = rng.normal(size=V.shape[1:]).astype(np.float32)
+    _, gw, gb = _gpu_grad(V, w, 0.1, r, K, every, lambda h, x: torch.from_numpy(c).cuda())
+    gwo, gbo = oracle.grad_csr(V.astype(np.float64), w.astype(np.float64), 0.1, 0.1, 1.0, r,
+                               np.ones(V[0].size), K, c.astype(np.float64))
+    scale = max(np.abs(gwo).max(), abs(gbo))
+    assert np.abs(gw - gwo).max() <= 2e-4 * scale
+    assert abs(gb - gbo) <= 2e-4 * scale
+
+
+def test_graph_replay_of_the_generic_stencil():
+    """Forward and reverse pass of a radius with rt = 3 replayed from CUDA graphs: what direct launches
+    give, to the order of the FP64 atomic sums."""
+    sf = _sf()
+    T, H, W, r = 6, 40, 70, (3, 1, 2)
+    V, _, w = synth.multichannel(T, H, W, C=3, seed=4011)
+    feats = torch.from_numpy(V).cuda()
+    c = torch.randn((T, H, W), device="cuda", generator=torch.Generator(device="cuda").manual_seed(3))
+    res = {}
+    for on in (False, True):
+        with sf.PowerIteration(3, T, H, W) as h:
+            h.enable_graphs(on)
+            h.set_features(feats, w, 0.2)
+            x = torch.empty((T, H, W), device="cuda")
+            for _ in range(3):
+                h.power_iterate(None, radius=r, iters=6, x=x)
+            h.power_iterate(feats, w, 0.2, r, iters=6, record_every=2)
+            for _ in range(3):
+                gw, gb = h.backward(c, r)
+            res[on] = (x.cpu().numpy(), np.append(gw, gb))
+    np.testing.assert_allclose(res[True][0], res[False][0], rtol=1e-6, atol=1e-9)
+    np.testing.assert_allclose(res[True][1], res[False][1], rtol=1e-6, atol=1e-9 * np.abs(res[False][1]).max())

@@ -81,3 +81,22 @@ def test_separate_maps_unsupported_paths(sf):
         with pytest.raises(sf.SFSegError) as e:
             h.power_iterate(None, radius=(1, 3, 3), iters=4, record_every=2)
         assert e.value.status == "UNSUPPORTED"
+
+
+@pytest.mark.parametrize("T,H,W,radius", [(24, 325, 449, (1, 3, 3)), (24, 325, 449, (2, 7, 7)), (24, 325, 449, (1, 6, 6)),
+                                          (5, 20, 33, (3, 2, 3)), (6, 20, 33, (4, 1, 2))])
+def test_separate_maps_on_every_kernel(sf, T, H, W, radius):
+    """The streaming kernel's separate-map form (own and padded radii) and the generic stencil's (rt = 3,
+    4), float32 to the roundings of 4 steps, 2^-24 each, and with two bf16 steps."""
+    rng = np.random.default_rng(T + sum(radius))
+    s, f = rng.random((2, T, H, W)).astype(np.float32)
+    iters = 4
+    xo, nuo = oracle.power_filter(s.astype(np.float64), f.astype(np.float64), 0.2, 1.0, radius, np.ones(s.shape), iters)
+    with sf.PowerIteration(1, T, H, W, p=0.2) as h:
+        h.set_features_sf(torch.from_numpy(s[None]).cuda(), None, 0.0, torch.from_numpy(f[None]).cuda())
+        x, nu = h.power_iterate(None, radius=radius, iters=iters, return_norms=True)
+        xb = h.power_iterate(None, radius=radius, iters=iters, iters_bf16=2)
+    tol = iters * (2 * sum(radius) + 3 + 12) * 2.0 ** -24
+    assert np.abs(x.cpu().numpy() - xo).max() <= tol * xo.max()
+    np.testing.assert_allclose(nu, nuo, rtol=tol)
+    assert np.abs(xb.cpu().numpy() - xo).max() <= 2e-2 * xo.max()

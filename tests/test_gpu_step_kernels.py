@@ -214,3 +214,27 @@ def test_unary_below_the_normal_range(sf, radius, T, H, W):
     xo, nuo = oracle.power_filter(f64, f64, 9.6, 1.0, radius, np.ones(f.shape), 3)
     assert np.abs(xi - xo).max() <= 3 * (2 * sum(radius) + 3 + 12) * 2.0 ** -24 * xo.max()
     np.testing.assert_allclose(nu, nuo, rtol=1e-5)
+
+
+@pytest.mark.parametrize("r", [(1, 3, 3), (2, 7, 7), (2, 4, 4)])
+def test_adjoint_on_the_streaming_kernel(sf, r):
+    """The recording, recomputing and reverse steps of the streaming kernel on radii of its own and a
+    padded one: as test_padded_radius_adjoint, four steps in two segments."""
+    T, H, W = 40, 325, 561
+    rng = np.random.default_rng(5)
+    V = rng.random((2, T, H, W)).astype(np.float32)
+    c = rng.normal(size=(T, H, W)).astype(np.float32)
+    w = np.array([0.8, -0.5], dtype=np.float32)
+    with sf.PowerIteration(2, T, H, W) as h:
+        h.power_iterate(torch.from_numpy(V).cuda(), w, 0.1, r, iters=4, record_every=2)
+        gw, gb = h.backward(torch.from_numpy(c).cuda(), r)
+    d = np.array([0.6, 0.8, -0.5])
+
+    def loss(t):
+        f = oracle.combine(V.astype(np.float64), w.astype(np.float64) + t * d[:2], 0.1 + t * d[2])
+        x, _ = oracle.power_filter(f, f, 0.1, 1.0, r, np.ones(f.shape), 4)
+        return float((x * c).sum())
+
+    num = (loss(1e-4) - loss(-1e-4)) / 2e-4
+    scale = float(np.abs(np.append(gw, gb)).max())
+    assert abs(gw[0] * d[0] + gw[1] * d[1] + gb * d[2] - num) <= 1e-4 * scale

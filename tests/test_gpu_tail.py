@@ -132,3 +132,21 @@ def test_stop_at_a_later_step_keeps_the_step_before(sf, T, H, W, radius, separat
             h.soft_binarize(y, radius, iters=4, gain=200.0, center=2.0, inplace=True)
         assert e.value.status == "ZERO_NORM"
         assert torch.equal(y, one)
+
+
+@pytest.mark.parametrize("shape,radius", [((5, 30, 40), (3, 1, 2)), ((6, 20, 33), (4, 3, 2)), ((9, 40, 150), (1, 6, 6)),
+                                          ((24, 325, 449), (1, 3, 3)), ((24, 325, 449), (2, 7, 7))])
+def test_soft_binarize_on_every_kernel(sf, shape, radius):
+    """The generic stencil (rt = 3, 4), a padded radius, and the streaming kernel with the maximum taken
+    in the step, three steps each, against the oracle."""
+    T, H, W = shape
+    V = synth.drifting_blob(T, H, W, seed=7300 + T)
+    f = V[0].astype(np.float64)
+    rng = np.random.default_rng(T)
+    x0 = rng.random(shape).astype(np.float32)
+    with sf.PowerIteration(1, T, H, W, p=0.3) as h:
+        h.set_features(torch.from_numpy(V).cuda())
+        x, mask = h.soft_binarize(torch.from_numpy(x0).cuda(), radius, iters=3, gain=6.0, center=0.4)
+        x, mask = x.cpu().numpy().astype(np.float64), mask.cpu().numpy()
+    xo, _ = oracle.soft_binarize(f, f, 0.3, 1.0, radius, x0.astype(np.float64), 3, 6.0, 0.4)
+    _check(x, mask, xo, margin=1e-4)
