@@ -164,11 +164,10 @@ bool launch_iterate_fast_last(const float* vin, float* x, const float* f, const 
     return run(args(kStepMax, vin, x, f, g, tp, inv_alpha, p, acc_in, acc_out, flags, s));
 }
 
-bool launch_iterate_fast_ckpt(const float* vin, void* out, bool out_x, const float* f, const Geom& g, const Taps& tp,
+bool launch_iterate_fast_ckpt(const float* vin, float* out, const float* f, const Geom& g, const Taps& tp,
                               float inv_alpha, float p, const double* acc_in, double* acc_out, float* ckpt, int* flags,
                               cudaStream_t s) {
     StepArgs a = args(kRecord, vin, out, f, g, tp, inv_alpha, p, acc_in, acc_out, flags, s);
-    a.out_x = out_x;
     a.out2 = ckpt;
     return run(a);
 }

@@ -190,17 +190,18 @@ bool launch_iterate(const void* vin, int vin_type, void* out, int out_type, bool
         note_step(true, tp, vin_type, out_type, "x~", ckpt != nullptr, false);
         return true;
     }
-    // The TMA kernel serves the method's radii, recording steps (float32, shared maps) included.
+    // The TMA kernels serve the radii that a compiled one covers, recording steps (float32, shared maps)
+    // included.
     if (ckpt == nullptr && fast_step_supported(tp) &&
         launch_iterate_fast(vin, vin_type, out, out_type, out_x, f, g, tp, inv_alpha, p, acc_in, acc_out, flags, s,
                             s32)) {
         note_step(true, tp, vin_type, out_type, caller_x, false, s32 != nullptr);
         return false;
     }
-    if (ckpt != nullptr && vin_type == kF32 && s32 == nullptr && fast_step_supported(tp) &&
-        launch_iterate_fast_ckpt((const float*)vin, out, out_x, (const float*)f, g, tp, inv_alpha, p, acc_in, acc_out,
+    if (ckpt != nullptr && !out_x && vin_type == kF32 && s32 == nullptr && fast_step_supported(tp) &&
+        launch_iterate_fast_ckpt((const float*)vin, (float*)out, (const float*)f, g, tp, inv_alpha, p, acc_in, acc_out,
                                  ckpt, flags, s)) {
-        note_step(true, tp, vin_type, out_type, caller_x, true, false);
+        note_step(true, tp, vin_type, out_type, nullptr, true, false);
         return false;
     }
     // Radii without a TMA kernel, or a tensor map the driver would not encode: the generic

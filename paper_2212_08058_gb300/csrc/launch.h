@@ -73,9 +73,10 @@ bool launch_iterate_fast_last(const float* vin, float* x, const float* f, const 
 // v = u x (internal layout) for a caller-layout x, u = s^p with s the unary map (s32, or f32).
 void launch_to_state(const float* x, const float* f32, const float* s32, float p, Geom g, float* v, cudaStream_t s);
 
-// The TMA step that also records x~_{k+1} (internal layout) into ckpt, float32 storage; false
-// (nothing launched) for a radius without a compiled kernel.
-bool launch_iterate_fast_ckpt(const float* vin, void* out, bool out_x, const float* f, const Geom& g, const Taps& tp,
+// The TMA step that also records x~_{k+1} (internal layout) into ckpt, float32 storage, not the last of a
+// call (its record is launch_iterate_fast_last's output); false (nothing launched) for a radius that no
+// compiled kernel covers.
+bool launch_iterate_fast_ckpt(const float* vin, float* out, const float* f, const Geom& g, const Taps& tp,
                               float inv_alpha, float p, const double* acc_in, double* acc_out, float* ckpt, int* flags,
                               cudaStream_t s);
 

@@ -77,9 +77,7 @@ bool step_dispatch(const StepArgs& a) {
             if (a.out_x) return K::template launch<bf, float, true, false, kStep>(a);
             return a.out_type == kBF16 ? K::template launch<bf, bf, false, false, kStep>(a)
                                        : K::template launch<bf, float, false, false, kStep>(a);
-        case kRecord:
-            return a.out_x ? K::template launch<float, float, true, false, kRecord>(a)
-                           : K::template launch<float, float, false, false, kRecord>(a);
+        case kRecord: return K::template launch<float, float, false, false, kRecord>(a);
         case kQPass: return K::template launch<float, float, false, false, kQPass>(a);
         case kGPass: return K::template launch<float, float, false, false, kGPass>(a);
         case kStepQ: return K::template launch<float, float, false, false, kStepQ>(a);
