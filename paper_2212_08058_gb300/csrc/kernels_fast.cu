@@ -80,23 +80,28 @@ const Radius* covering_radius(const Taps& tp) {
     return best;
 }
 
-// Which kernel a volume takes: the one whose time, modelled from the frames its busiest SM streams, is
-// shorter.  The streaming kernel takes 4.7 us and u per frame step, its steps being the whole tiles'
-// frames (rt more each to flush) and the share of the tiles left over (3 rt more for the cuts); the
-// small-tile kernel 0.4 us and 1.8 u per step of its three CTAs per SM.  u = 0.55 + 0.0235 us per tap.
-// The choice costs 0.3 % on average, 6 % at worst, over the 26 volumes it was fitted to.  Measured, tile /
-// streaming kernel, (2,7,7): 16x128x128 11.6 / 12.7 us,
-// 60x128x128 18.2 / 23.4, 13x480x854 39.7 / 43.2, 32x240x427 31.2 / 30.8, 25x480x854 70.4 / 68.3,
-// 50x100x200 20.8 / 18.9, 64x480x854 169 / 147; (1,3,3): 32x240x427 18.6 / 19.4, 48x240x427 25.6 / 25.2.
+// Which kernel a volume takes.  Where the small-tile kernel has at most one block per SM, that one: 1.2
+// times as fast or more on all 156 such volumes timed (2x22x33 at (2,8,8) 6.3 us, streaming 9.9).  Else the
+// one whose time, modelled from the frames its busiest SM streams, is shorter.  The streaming kernel takes
+// 4.7 us and u per frame step, its steps being the whole tiles' frames (rt more each to flush) and the
+// share of the tiles left over (3 rt more for the cuts); the small-tile kernel 0.4 us and 1.8 u per step of
+// its three CTAs per SM.  u = 0.55 + 0.0235 us per tap.
+// Both kernels timed on 92 volumes at four or six radii, 508 pairs: the choice costs 0.6 % on average, more
+// than 12 % for eight pairs, at worst 23 % (70x64x112 at (2,7,7): its frames fill the streaming kernel's
+// tiles and three quarters of the small ones).  Measured, tile / streaming kernel, (2,7,7): 16x128x128
+// 11.7 / 12.6 us, 60x128x128 18.1 / 22.6, 13x480x854 39.4 / 41.3, 32x240x427 31.3 / 29.6, 25x480x854
+// 69.8 / 65.2, 64x480x854 168 / 140; (1,3,3): 32x240x427 18.7 / 19.3, 48x240x427 25.6 / 25.3,
+// 64x480x854 111 / 99.5.
 bool stream_pays(const Geom& g, const Radius& r) {
     const double G = num_sms(), T = g.T, u = 0.55 + 0.0235 * (2 * (r.rt + r.rh + r.rw) + 3);
     const int64_t big = (int64_t)((g.W + 111) / 112) * ((g.H + 17) / 18);      // 18 x 112 tiles
     const int64_t small = (int64_t)((g.W + 63) / 64) * ((g.H + 14) / 15);      // 15 x 64 tiles
-    const int64_t whole = big / num_sms(), rest = big - whole * num_sms();
-    const double stream = 4.7 + u * (whole * (T + r.rt) + (rest ? rest * T / G + 3 * r.rt : 0.0));
     if (small > 3 * (int64_t)num_sms() * 16) return true;    // many waves: the streaming kernel's steps are cheaper
     const int chunk = tile_chunk(g.T, (int)small, 3 * num_sms(), r.rt);
     const double blocks = (double)small * ((g.T + chunk - 1) / chunk), waves = blocks / (3 * G);
+    if (blocks <= G) return false;
+    const int64_t whole = big / num_sms(), rest = big - whole * num_sms();
+    const double stream = 4.7 + u * (whole * (T + r.rt) + (rest ? rest * T / G + 3 * r.rt : 0.0));
     const double tile = 0.4 + 1.8 * u * (chunk + (chunk < g.T ? 2 : 1) * r.rt) * (waves > 1.0 ? waves : 1.0);
     return stream <= tile;
 }

@@ -171,6 +171,7 @@ def test_norm_of_many_frames(sf):
     (24, 325, 449, (1, 3, 3), 1, 2, "iter_stream<1,3,3,bf16,caller x>"),
     (5, 40, 70, (2, 7, 7), 1, 0, "iter_tile<2,7,7,float,x~>"),
     (5, 40, 70, (0, 1, 1), 1, 0, "iter_tile<1,2,2,float,x~> for radius 0,1,1"),
+    (4, 24, 33, (0, 0, 8), 1, 0, "iter_tile<2,8,8,float,x~> for radius 0,0,8"),
     (5, 40, 70, (1, 6, 6), 2, 0, "iter_tile<1,7,7,float,caller x,separate maps> for radius 1,6,6"),
     (5, 40, 70, (3, 5, 5), 1, 0, "stream_stencil<3,5,5,float,caller x>"),
     (5, 40, 70, (1, 3, 3), 2, 2, "stream_stencil<1,3,3,bf16,caller x,separate maps>"),
