@@ -804,8 +804,9 @@ int sfseg_power_iterate_exact(sfseg_handle* h, const sfseg_neighborhood* nb, int
     SFSEG_CUDA(cudaMemsetAsync(acc, 0, sizeof(double) * (iters + 1), s));
     const float inv_alpha = (float)(1.0 / h->alpha);
     const float* x_user = init == SFSEG_INIT_USER ? x_inout : nullptr;
-    if (iters == 0) {   // x0 itself, normalised
-        if (!x_user) launch_fill(x_inout, h->N, 1.f, s);
+    if (iters == 0 && !x_user) {   // the uniform x0, normalised
+        launch_fill(x_inout, h->N, (float)(1.0 / std::sqrt((double)h->N)), s);
+    } else if (iters == 0) {
         launch_sumsq(x_inout, h->N, acc, s);
     } else {
         const ExactVolumes e = exact_volumes(h, center, s);
@@ -817,7 +818,7 @@ int sfseg_power_iterate_exact(sfseg_handle* h, const sfseg_neighborhood* nb, int
             else launch_exact_out(e.S, e.A, inv_alpha, h->g, x_inout, acc + iters, s);
         }
     }
-    launch_scale_inv_norm(x_inout, h->N, acc + iters, h->flags, s);
+    if (iters > 0 || x_user) launch_scale_inv_norm(x_inout, h->N, acc + iters, h->flags, s);
     SFSEG_LAUNCHED();
     if (norms_out) {
         std::vector<double> a((size_t)iters + 1);

@@ -161,3 +161,23 @@ def test_every_output_keeps_its_digits(sf, alpha):
         terms += 1
     bound = (2 * sum(r) + 3 + 2 * terms + 12 + 4 * alpha) * 2.0 ** -24 * (math.e if alpha <= 1.0 else 1.0)
     assert (np.abs(y - yo) / yo).max() <= bound
+
+
+@pytest.mark.parametrize("T,H,W", [(1, 1, 1), (3, 17, 41), (2, 480, 854)])
+def test_no_exact_steps_is_the_normalised_start(sf, T, H, W):
+    """iters = 0: the uniform vector of norm 1 (each component a rounded N^-1/2), or the caller's x over
+    its norm (2 roundings), and a zero x is reported."""
+    V = torch.rand((1, T, H, W), device="cuda") + 0.1
+    x = torch.rand((T, H, W), device="cuda") + 0.1
+    with sf.PowerIteration(1, T, H, W) as h:
+        h.set_features(V)
+        u = h.power_iterate_exact((1, 3, 3), iters=0)
+        assert float((u.double() * (T * H * W) ** 0.5 - 1.0).abs().max()) <= 2.0 ** -24
+        n0 = sf.kernel_launches()
+        h.power_iterate_exact((1, 3, 3), iters=0, x=u)
+        assert sf.kernel_launches() - n0 == 2          # f's range, and the vector
+        y = h.power_iterate_exact((1, 3, 3), iters=0, x=x.clone(), init="user").double()
+        assert float((y / (x.double() / x.double().norm()) - 1.0).abs().max()) <= 4 * 2.0 ** -24
+        with pytest.raises(sf.SFSegError) as e:
+            h.power_iterate_exact((1, 3, 3), iters=0, x=torch.zeros_like(x), init="user", return_norms=True)
+        assert e.value.status == "ZERO_NORM"
