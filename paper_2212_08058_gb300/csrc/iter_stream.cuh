@@ -635,7 +635,7 @@ static bool launch_t(const StepArgs& a) {
     if (!OUT_X && !make_step_map(&M.out, a.out, sizeof(TVO) == 2, g, TW, TH)) return false;
     if (E::OUT2 && !make_step_map(&M.out2, a.out2, false, g, TW, TH)) return false;
     auto kern = iter_stream<RT, RH, RW, TS, TVO, OUT_X, SEP, MODE>;
-    static unsigned long long attr_set = 0;   // devices on which the attribute is set
+    static std::atomic<unsigned long long> attr_set{0};   // devices on which the attribute is set
     if (!(attr_set & device_bit())) {
         if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM) != cudaSuccess) return false;
         attr_set |= device_bit();

@@ -440,8 +440,8 @@ static bool launch_t(const StepArgs& a) {
     CUtensorMap mv, mf;
     if (!make_step_map(&mv, a.vin, bf, g, BW, C::BH) || !make_step_map(&mf, a.f, bf, g, BW, C::BH)) return false;
     auto kern = iter_tile<RT, RH, RW, TS, TVO, OUT_X, SEP, MODE>;
-    static int slots_per_sm = -1;
-    static unsigned long long attr_set = 0;   // devices on which the attribute is set
+    static std::atomic<int> slots_per_sm{1};
+    static std::atomic<unsigned long long> attr_set{0};   // devices on which the attribute is set
     if (!(attr_set & device_bit())) {
         if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM) != cudaSuccess) return false;
         int nb = 0;

@@ -149,14 +149,13 @@ void count_launches(int n) { g_launches.fetch_add(n, std::memory_order_relaxed);
 int64_t launches_so_far() { return g_launches.load(std::memory_order_relaxed); }
 
 int num_sms() {
-    static int n = 0;
-    if (n == 0) {
-        int dev = 0;
+    static const int sms = [] {
+        int dev = 0, n = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-        if (n <= 0) n = 1;
-    }
-    return n;
+        return n > 0 ? n : 1;
+    }();
+    return sms;
 }
 
 template <typename TVI, typename TVO, typename TF, bool OUT_X>

@@ -1081,17 +1081,14 @@ typedef CUresult (*EncodeFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void
                              CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
 EncodeFn encode() {
-    static EncodeFn fn = nullptr;
-    static bool tried = false;
-    if (!tried) {
-        tried = true;
+    static const EncodeFn fn = [] {   // once, whichever thread comes first
         void* p = nullptr;
         cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) ==
-                cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            fn = (EncodeFn)p;
-    }
+        const bool ok = cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) ==
+                            cudaSuccess &&
+                        q == cudaDriverEntryPointSuccess;
+        return ok ? (EncodeFn)p : nullptr;
+    }();
     return fn;
 }
 
@@ -1194,7 +1191,7 @@ int launch_conv(const void* in, int T, int H, int W, const ConvArgs& a, int item
     CUtensorMap m;
     if (!act_map(&m, in, CIN, T, H, W, RW, 1, Cf::NF)) return nfail(SFSEG_ERR_CUDA, "tensor map encoding failed");
     auto k = conv3d_tc<CIN, COUT, EPI, FR>;
-    static unsigned long long attr_set = 0;   // devices on which the attribute is set
+    static std::atomic<unsigned long long> attr_set{0};   // devices on which the attribute is set
     if (!(attr_set & device_bit())) {
         NET_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, Cf::SMEM));
         attr_set |= device_bit();
@@ -1241,7 +1238,7 @@ int launch_last(const __nv_bfloat16* in, int T, int H, int W, const LastArgs& a,
     using L = LastCfg<FR>;
     CUtensorMap m;
     if (!act_map(&m, in, 32, T, H, W, RW, 1, L::NF)) return nfail(SFSEG_ERR_CUDA, "tensor map encoding failed");
-    static unsigned long long attr_set = 0;   // devices on which the attribute is set
+    static std::atomic<unsigned long long> attr_set{0};   // devices on which the attribute is set
     if (!(attr_set & device_bit())) {
         NET_CUDA(cudaFuncSetAttribute(conv_last_tc<FR>, cudaFuncAttributeMaxDynamicSharedMemorySize, L::SMEM));
         attr_set |= device_bit();
@@ -1354,7 +1351,7 @@ int run_wgrad(sfseg_net* n, int cout, int cin, const __nv_bfloat16* dz, const __
         return nfail(SFSEG_ERR_CUDA, "tensor map encoding failed");
     if (!n->wg_part) NET_CUDA(cudaMalloc(&n->wg_part, (size_t)num_sms() * WgCfg<4, 4>::PART * sizeof(float)));
     auto k = wgrad_tc<NCI, NCO>;
-    static unsigned long long attr_set = 0;   // devices on which the attribute is set
+    static std::atomic<unsigned long long> attr_set{0};   // devices on which the attribute is set
     if (!(attr_set & device_bit())) {
         NET_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, Cf::SMEM));
         attr_set |= device_bit();

@@ -131,7 +131,7 @@ static void run_stencil(const Op& op, const Taps& tp, int TH, const double* acc_
                         double* acc_out2, int* flags, cudaStream_t s) {
     const Geom& g = op.g;
     const size_t smem = stencil_smem(Op::NS, TH, tp);
-    static bool attr_set = false;   // one per Op instantiation
+    static std::atomic<bool> attr_set{false};   // one per Op instantiation
     if (!attr_set) {
         cudaFuncSetAttribute(stream_stencil<Op>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
         attr_set = true;
