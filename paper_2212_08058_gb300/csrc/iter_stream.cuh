@@ -1,41 +1,39 @@
 // iter_stream.cuh -- the power-iteration step of Eq. 7 with a compiled radius, written for sm_103a:
 // the kernel for all but small volumes (those: iter_tile.cuh).
 //
-// One persistent CTA per SM (12 warps) streams frames of 18 x 112 tiles of (h, w) along t.  Its
-// warps have two roles that run at the same time, connected by rings in shared memory:
+// One persistent CTA per SM (16 warps: 4 h-pass, 8 w-pass, 4 for copies and the norm) streams frames of
+// 18 x 112 tiles of (h, w) along t.  Its warps have roles that run at the same time, connected by rings in
+// shared memory:
 //   - Copies.  One thread keeps TMA copies of the raw halo boxes of v (= u x~) and f (18 + 2rh rows
 //     of 128 columns) in flight, three frames deep; zero fill outside the volume is the zero padding,
 //     also for whole frames after the last.
 //   - h-pass, warps 0..3: a thread takes a column pair and 9 output rows (64 pairs x 2 row groups);
-//     it walks down the 9 + 2rh input rows once, forms the three signals z1 = v, z2 = f^2 v,
-//     z3 = f v of each, and accumulates them into its 9 x 3 outputs with packed FP32 FMAs (FFMA2,
-//     one per column pair).  The result goes to a ring of two frames of [3][18][132] floats.
-//   - w-pass, warps 4..11: a thread takes 8 output columns of one row (14 x 18 = 252 of 256
-//     threads); it loads its window of the h-pass result as 16-byte pieces (the odd taps run as
-//     two scalar FMAs: rebuilding their pairs for packed ones costs more moves) and feeds the three w-filtered signals straight into the t-filter, kept in registers in transposed
-//     direct form (2rt running partial sums per value, no frame ring to index).
+//     it walks down the 9 + 2rh input rows once, each loaded a row ahead, forms the three signals z1 = v,
+//     z2 = f^2 v, z3 = f v of each, and accumulates them into its 9 x 3 outputs with packed FP32 FMAs
+//     (FFMA2, one per column pair).  The result goes to a ring of two frames of [3][18][132] floats.
+//   - w-pass, warps 4..11: a thread takes 8 output columns of one row (14 x 18 = 252 of 256 threads); it
+//     loads its window of the h-pass result as 16-byte pieces (the odd taps run as two scalar FMAs:
+//     rebuilding their pairs for packed ones costs more moves) and feeds the three w-filtered signals
+//     straight into the t-filter, kept in registers in transposed direct form (2rt running partial sums
+//     per value, no frame ring to index).
 //   - Epilogue, same threads: Eq. 7 combination for the frame rt behind, with f of that frame from a
 //     TMA-fed tile, the Eq. 8 norm partial, and the next state into a tile that a TMA store writes
 //     out (which clips at the volume's edges, so no lane tests its column).
 // Every hand-over is an mbarrier of the ring slot concerned: no barrier stops all warps.
 //
-// Why this shape.  The step is bound by the FP32 pipe (105 FMA per voxel at (2,7,7) against 12
-// bytes), so what counts is the work that is not algorithmic and the time the pipe idles.  The
-// kernel before this one (iter_tile.cuh, which small volumes still take) runs three CTAs of 4 warps
-// per SM, each a 15 x 64 tile, all warps doing the h-pass and then the w-pass between CTA barriers:
-// 80 columns h-filtered for 64 (here 128 for 112), 19 input rows read and multiplied per 5 output
-// rows (here 23 per 9), and, with one wave of CTAs, the three CTAs of an SM ended at 121, 145 and
-// 175 us (the oldest is favoured), the last one running alone.
-// Two facts of the instruction set decide the rest.  A packed FMA takes 3 clocks when its three
-// register pairs are all new and 2 when one is a constant or was read by the instruction before it
-// (measured): taps stay in the parameter constants.  And a shared-memory pointer rounded up through
-// an integer loses its address space: every access was a generic one until the alignment became an
-// offset (184 -> 152 us per step here, 180 -> 172 in the older kernel).
-// Three smaller ones: the odd taps of the w-pass as scalar FMAs and the next input row of the h-pass
-// loaded a row ahead (147.6 -> 138.7 us together), and 184 / 112 / 32 registers for the w-pass, the
-// h-pass and the copy threads (192 / 96 / 32: 138.7, now 137.7).
-// Measured per step, before -> now: (2,7,7) 64x480x854 180.5 -> 138.2 us (the algorithmic
-// multiply-adds alone 68 us), 120x1080x1920 1465 -> 1163; (1,3,3) 64x480x854 123 -> 94.6.
+// Why this shape.  The step is bound by the FP32 pipe (105 FMA per voxel at (2,7,7) against 12 bytes), so
+// what counts is the work that is not algorithmic and the time the pipe idles.  Against the small-volume
+// kernel's three CTAs of 4 warps per SM, each on a 15 x 64 tile with all warps doing the h-pass and then
+// the w-pass between CTA barriers: 128 columns are h-filtered for 112 (there 80 for 64), 23 input rows read
+// and multiplied per 9 output rows (there 19 per 5), and an SM's work ends at one time (there the oldest
+// of its CTAs is favoured and the last runs alone: 121, 145 and 175 us in one wave).
+// Two facts of the instruction set decide the rest.  A packed FMA takes 3 clocks when its three register
+// pairs are all new and 2 when one is a constant or was read by the instruction before it (measured): taps
+// stay in the parameter constants.  And a shared-memory pointer rounded up through an integer loses its
+// address space, so that every access is a generic one: the alignment is an offset (152 us per step; 184
+// through an integer).
+// Measured per step, small-volume kernel / this one: (2,7,7) 64x480x854 168 / 138 us (the algorithmic
+// multiply-adds alone 68 us), 120x1080x1920 1163 here; (1,3,3) 64x480x854 111 / 95.
 #pragma once
 
 #include "order_key.cuh"
@@ -425,13 +423,20 @@ iter_stream(const __grid_constant__ Maps M, const __grid_constant__ Params P) {
         // 2rt running partial sums of the 2rt+1-tap filter; with x[n] the w-filtered frame n and
         // g_j = gt[2rt - j], the output y[n] = sum_j g_j x[n - j] is the t-filtered frame n - rt.
         float2 st[2 * RT > 0 ? 2 * RT : 1][3][4];
-        // The norm (or dot product): kFold output frames in float32, those sums in FP64 in shared memory.
-        // One float32 sum over a long run loses digits: 500 equal frames put the norm 1.2e-5 off, where
-        // 128 squares per sum are at most 3.8e-6 away.  The fold stands with the output frame's inputs, where
-        // it costs nothing (50 steps at 480p 7391 us); around the frame loop they took 7419, at its head 7435,
-        // and a step with the fold at the frame's end 144 us against 138.
+        // The norm (or dot product): kFold frames in float32, those sums in FP64 in shared memory.  One
+        // float32 sum over a long run loses digits: 500 equal frames put the norm 1.2e-5 off, where 128
+        // squares per sum are at most 3.8e-6 away.  Where the fold stands decides the compiler's schedule of
+        // the passes: for rw >= 7 with the output frame's inputs, else around the frame loop.  480p, us per
+        // step, inside / around: (1,3,3) 97.5 / 94.0, (2,3,3) 107.0 / 105.0, (1,7,7) 130.2 / 134.3, (2,8,8)
+        // 150.3 / 156.2, (2,7,7) 138.1 / 138.7 (in bf16 147 / 151); at the frame's end or after its passes
+        // it is never better than both.
         float2 part = make_float2(0.f, 0.f);
         red[i] = 0.0;
+        auto fold = [&] {
+            red[i] += (double)part.x + (double)part.y;
+            part = make_float2(0.f, 0.f);
+        };
+        constexpr bool kFoldInside = RW >= 7;
         float tmax = 0.f;   // MODE 8: the largest output so far (outputs are >= 0)
         const int tile_off = row * TW + seg * 8;
 
@@ -444,164 +449,174 @@ iter_stream(const __grid_constant__ Maps M, const __grid_constant__ Params P) {
                 for (int k = 0; k < 3; ++k)
 #pragma unroll
                     for (int m = 0; m < 4; ++m) st[a][k][m] = make_float2(0.f, 0.f);
+            int to = max(r.t0 - RT, 0) - RT;   // output frame of each step
+            auto frames = [&](int end) {
 #pragma unroll 1
-            for (int to = max(r.t0 - RT, 0) - RT; to < r.t1; ++to) {   // output frame of each step
-                // ---------------- the output frame's inputs, while the h-pass is still at work
-                const bool emit = to >= r.t0;
-                const int b = e & 1;
-                float2 fo[4], so[4], uo[4];
-                if (emit) {
-                    if (e % kFold == 0) {
-                        red[i] += (double)part.x + (double)part.y;
-                        part = make_float2(0.f, 0.f);
-                    }
-                    const uint32_t ph = (uint32_t)(e >> 1) & 1;
-                    ok = mbar_wait_bounded(&ffull[b], ph) && (e < 2 || mbar_wait_bounded(&oempty[b], ph ^ 1));
-                    ld_cols(reinterpret_cast<const TS*>(smem + C::O_F + b * C::FT) + tile_off, fo);
-                    if constexpr (E::IN2)
-                        ld_cols(reinterpret_cast<const float*>(smem + C::O_I2 + b * C::T32) + tile_off, so);
-#pragma unroll
-                    for (int m = 0; m < 4; ++m) {
-                        const float2 sv = SEP ? so[m] : fo[m];
-                        uo[m] = make_float2(unary_pow_fast<true>(sv.x, P.p), unary_pow_fast<true>(sv.y, P.p));
-                    }
-                    // again for the rest, in a branch never taken for the usual p: the longer form
-                    // throughout costs 1.4 % (solve 480p 7391 -> 7495 us)
-                    if (P.p > kUnaryFtzP) {
+                for (; to < end; ++to) {
+                    // ---------------- the output frame's inputs, while the h-pass is still at work
+                    const bool emit = to >= r.t0;
+                    const int b = e & 1;
+                    float2 fo[4], so[4], uo[4];
+                    if (emit) {
+                        if constexpr (kFoldInside)
+                            if (e % kFold == 0) fold();
+                        const uint32_t ph = (uint32_t)(e >> 1) & 1;
+                        ok = mbar_wait_bounded(&ffull[b], ph) && (e < 2 || mbar_wait_bounded(&oempty[b], ph ^ 1));
+                        ld_cols(reinterpret_cast<const TS*>(smem + C::O_F + b * C::FT) + tile_off, fo);
+                        if constexpr (E::IN2)
+                            ld_cols(reinterpret_cast<const float*>(smem + C::O_I2 + b * C::T32) + tile_off, so);
 #pragma unroll
                         for (int m = 0; m < 4; ++m) {
                             const float2 sv = SEP ? so[m] : fo[m];
-                            uo[m] = make_float2(unary_pow_fast(sv.x, P.p), unary_pow_fast(sv.y, P.p));
+                            uo[m] = make_float2(unary_pow_fast<true>(sv.x, P.p), unary_pow_fast<true>(sv.y, P.p));
                         }
-                    }
-                }
-                ok = ok && mbar_wait_bounded(&qfull[q], qp);
-                if (!__all_sync(0xffffffffu, ok)) {
-                    ok = false;
-                    break;
-                }
-                // ---------------- w-pass: Q -> x[n], then the t-filter update
-                float2 y[3][4];
-                if (item) {
-                    const float* Q = reinterpret_cast<const float*>(smem + C::O_Q + q * C::Q) + row * QP + PADW +
-                                     seg * 8 - C::OFF;
-#pragma unroll
-                    for (int k = 0; k < 3; ++k) {
-                        float2 acc[4];   // four independent chains (one per column pair)
-#pragma unroll
-                        for (int m = 0; m < 4; ++m) acc[m] = make_float2(0.f, 0.f);
-                        float2 pa[C::NPAIR];
-#pragma unroll
-                        for (int j = 0; j < C::NPAIR / 2; ++j) {
-                            const float4 a = reinterpret_cast<const float4*>(Q + k * TH * QP)[j];
-                            pa[2 * j] = make_float2(a.x, a.y);
-                            pa[2 * j + 1] = make_float2(a.z, a.w);
-                        }
-#pragma unroll
-                        for (int d = 0; d <= 2 * RW; ++d) {
-                            const float2 gd = gwr[off(d, RW)];
+                        // again for the rest, in a branch never taken for the usual p: the longer form
+                        // throughout costs 1.4 % (solve 480p 7391 -> 7495 us)
+                        if (P.p > kUnaryFtzP) {
 #pragma unroll
                             for (int m = 0; m < 4; ++m) {
-                                const int c = 2 * m + d + C::OFF - RW;
-                                if (c & 1) {   // odd-aligned pair: two scalar FMAs
-                                    acc[m].x = fmaf(pa[c >> 1].y, gd.x, acc[m].x);
-                                    acc[m].y = fmaf(pa[(c >> 1) + 1].x, gd.x, acc[m].y);
-                                } else {
-                                    acc[m] = fma2(pa[c >> 1], gd, acc[m]);
-                                }
-                            }
-                        }
-#pragma unroll
-                        for (int m = 0; m < 4; ++m) {
-                            const float2 x = acc[m];
-                            if constexpr (RT == 0) {
-                                y[k][m] = mul2(x, gtr[0]);
-                            } else {
-                                y[k][m] = fma2(x, gtr[RT], st[0][k][m]);
-#pragma unroll
-                                for (int j = 0; j < 2 * RT - 1; ++j)
-                                    st[j][k][m] = fma2(x, gtr[off(2 * RT - 1 - j, RT)], st[j + 1][k][m]);
-                                st[2 * RT - 1][k][m] = mul2(x, gtr[RT]);
+                                const float2 sv = SEP ? so[m] : fo[m];
+                                uo[m] = make_float2(unary_pow_fast(sv.x, P.p), unary_pow_fast(sv.y, P.p));
                             }
                         }
                     }
-                }
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&qempty[q]);
-                if (++q == NQ) q = 0, qp ^= 1;
-                if (!emit) continue;
-                // ---------------- Eq. 7 combination for frame to
-                if (item) {
-                    float2 outv[4], outq[4];
-#pragma unroll
-                    for (int m = 0; m < 4; ++m) {
-                        const float2 fv = fo[m];
-                        const float2 u = uo[m];
-                        const float2 ee = fma2(make_float2(-fv.x, -fv.y), fv, f2(P.inv_alpha));   // 1/alpha - f^2
-                        if constexpr (MODE == 7) {
-                            float2 F = make_float2(1.f, 1.f);
-                            const float2 f3 = mul2(fv, mul2(fv, fv));
-                            for (int i3 = 0; i3 < P.exj; ++i3) F = mul2(F, f3);
-                            const float2 inner = fma2(mul2(fv, f2(P.exc[2])), y[1][m], mul2(f2(P.exc[1]), y[2][m]));
-                            outv[m] = mul2(mul2(s2, F), fma2(fv, inner, mul2(f2(P.exc[0]), y[0][m])));
-                            if (P.exj > 0) outv[m] = __fadd2_rn(outv[m], so[m]);   // the terms so far
-                        } else if constexpr (MODE == 0 || MODE == 4 || MODE == 6 || MODE == 8) {
-                            float2 B = fma2(ee, y[0][m], make_float2(-y[1][m].x, -y[1][m].y));
-                            B = fma2(mul2(f2(2.f), fv), y[2][m], B);
-                            const float2 xt = mul2(mul2(s2, u), B);
-                            part = fma2(xt, xt, part);
-                            if constexpr (MODE == 8) tmax = fmaxf(tmax, fmaxf(xt.x, xt.y));
-                            outv[m] = (OUT_X || MODE == 8) ? xt : mul2(u, xt);
-                            if constexpr (MODE == 4) outq[m] = xt;
-                            if constexpr (MODE == 6) {
-                                const float2 a1 = fma2(f2(P.p), ee, mul2(f2(-2.f), mul2(fv, fv)));
-                                const float2 a3 = mul2(f2(2.f * (P.p + 1.f)), fv);
-                                const float2 Qd = fma2(a1, y[0][m], mul2(f2(-P.p), y[1][m]));
-                                outq[m] = mul2(s2, fma2(a3, y[2][m], Qd));
-                            }
-                        } else {
-                            const float2 a1 = fma2(f2(P.p), ee, mul2(f2(-2.f), mul2(fv, fv)));
-                            const float2 a3 = mul2(f2(2.f * (P.p + 1.f)), fv);
-                            float2 Qd = fma2(a1, y[0][m], mul2(f2(-P.p), y[1][m]));
-                            Qd = mul2(s2, fma2(a3, y[2][m], Qd));
-                            if constexpr (MODE == 1) {
-                                outv[m] = Qd;
-                            } else {
-                                float2 B = fma2(ee, y[0][m], make_float2(-y[1][m].x, -y[1][m].y));
-                                B = fma2(mul2(f2(2.f), fv), y[2][m], B);
-                                outv[m] = mul2(mul2(u, u), B);
-                                part = fma2(so[m], B, part);
-                                outq[m] = Qd;
-                            }
-                        }
+                    ok = ok && mbar_wait_bounded(&qfull[q], qp);
+                    if (!__all_sync(0xffffffffu, ok)) {
+                        ok = false;
+                        break;
                     }
-                    if constexpr (OUT_X) {
-                        // caller layout: rows of W values, 8-byte aligned when W is even (and the
-                        // caller's base is), then one 8-byte store per pair
-                        const Geom& g = P.g;
-                        const int h = r.h0 + row, wb = r.w0 + seg * 8;
-                        float* o = reinterpret_cast<float*>(P.out) + ((int64_t)to * g.H + h) * g.W + wb;
-                        if (h < g.H) {
-                            if (wb + 8 <= g.W && (reinterpret_cast<uintptr_t>(o) & 7) == 0) {
+                    // ---------------- w-pass: Q -> x[n], then the t-filter update
+                    float2 y[3][4];
+                    if (item) {
+                        const float* Q = reinterpret_cast<const float*>(smem + C::O_Q + q * C::Q) + row * QP + PADW +
+                                         seg * 8 - C::OFF;
 #pragma unroll
-                                for (int m = 0; m < 4; ++m) reinterpret_cast<float2*>(o)[m] = outv[m];
-                            } else {
+                        for (int k = 0; k < 3; ++k) {
+                            float2 acc[4];   // four independent chains (one per column pair)
+#pragma unroll
+                            for (int m = 0; m < 4; ++m) acc[m] = make_float2(0.f, 0.f);
+                            float2 pa[C::NPAIR];
+#pragma unroll
+                            for (int j = 0; j < C::NPAIR / 2; ++j) {
+                                const float4 a = reinterpret_cast<const float4*>(Q + k * TH * QP)[j];
+                                pa[2 * j] = make_float2(a.x, a.y);
+                                pa[2 * j + 1] = make_float2(a.z, a.w);
+                            }
+#pragma unroll
+                            for (int d = 0; d <= 2 * RW; ++d) {
+                                const float2 gd = gwr[off(d, RW)];
 #pragma unroll
                                 for (int m = 0; m < 4; ++m) {
-                                    if (wb + 2 * m < g.W) o[2 * m] = outv[m].x;
-                                    if (wb + 2 * m + 1 < g.W) o[2 * m + 1] = outv[m].y;
+                                    const int c = 2 * m + d + C::OFF - RW;
+                                    if (c & 1) {   // odd-aligned pair: two scalar FMAs
+                                        acc[m].x = fmaf(pa[c >> 1].y, gd.x, acc[m].x);
+                                        acc[m].y = fmaf(pa[(c >> 1) + 1].x, gd.x, acc[m].y);
+                                    } else {
+                                        acc[m] = fma2(pa[c >> 1], gd, acc[m]);
+                                    }
+                                }
+                            }
+#pragma unroll
+                            for (int m = 0; m < 4; ++m) {
+                                const float2 x = acc[m];
+                                if constexpr (RT == 0) {
+                                    y[k][m] = mul2(x, gtr[0]);
+                                } else {
+                                    y[k][m] = fma2(x, gtr[RT], st[0][k][m]);
+#pragma unroll
+                                    for (int j = 0; j < 2 * RT - 1; ++j)
+                                        st[j][k][m] = fma2(x, gtr[off(2 * RT - 1 - j, RT)], st[j + 1][k][m]);
+                                    st[2 * RT - 1][k][m] = mul2(x, gtr[RT]);
                                 }
                             }
                         }
-                    } else {
-                        st_cols(reinterpret_cast<TVO*>(smem + C::O_O + b * C::OT) + tile_off, outv);
                     }
-                    if constexpr (E::OUT2) st_cols(reinterpret_cast<float*>(smem + C::O_O2 + b * C::T32) + tile_off, outq);
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&qempty[q]);
+                    if (++q == NQ) q = 0, qp ^= 1;
+                    if (!emit) continue;
+                    // ---------------- Eq. 7 combination for frame to
+                    if (item) {
+                        float2 outv[4], outq[4];
+#pragma unroll
+                        for (int m = 0; m < 4; ++m) {
+                            const float2 fv = fo[m];
+                            const float2 u = uo[m];
+                            const float2 ee = fma2(make_float2(-fv.x, -fv.y), fv, f2(P.inv_alpha));   // 1/alpha - f^2
+                            if constexpr (MODE == 7) {
+                                float2 F = make_float2(1.f, 1.f);
+                                const float2 f3 = mul2(fv, mul2(fv, fv));
+                                for (int i3 = 0; i3 < P.exj; ++i3) F = mul2(F, f3);
+                                const float2 inner = fma2(mul2(fv, f2(P.exc[2])), y[1][m], mul2(f2(P.exc[1]), y[2][m]));
+                                outv[m] = mul2(mul2(s2, F), fma2(fv, inner, mul2(f2(P.exc[0]), y[0][m])));
+                                if (P.exj > 0) outv[m] = __fadd2_rn(outv[m], so[m]);   // the terms so far
+                            } else if constexpr (MODE == 0 || MODE == 4 || MODE == 6 || MODE == 8) {
+                                float2 B = fma2(ee, y[0][m], make_float2(-y[1][m].x, -y[1][m].y));
+                                B = fma2(mul2(f2(2.f), fv), y[2][m], B);
+                                const float2 xt = mul2(mul2(s2, u), B);
+                                part = fma2(xt, xt, part);
+                                if constexpr (MODE == 8) tmax = fmaxf(tmax, fmaxf(xt.x, xt.y));
+                                outv[m] = (OUT_X || MODE == 8) ? xt : mul2(u, xt);
+                                if constexpr (MODE == 4) outq[m] = xt;
+                                if constexpr (MODE == 6) {
+                                    const float2 a1 = fma2(f2(P.p), ee, mul2(f2(-2.f), mul2(fv, fv)));
+                                    const float2 a3 = mul2(f2(2.f * (P.p + 1.f)), fv);
+                                    const float2 Qd = fma2(a1, y[0][m], mul2(f2(-P.p), y[1][m]));
+                                    outq[m] = mul2(s2, fma2(a3, y[2][m], Qd));
+                                }
+                            } else {
+                                const float2 a1 = fma2(f2(P.p), ee, mul2(f2(-2.f), mul2(fv, fv)));
+                                const float2 a3 = mul2(f2(2.f * (P.p + 1.f)), fv);
+                                float2 Qd = fma2(a1, y[0][m], mul2(f2(-P.p), y[1][m]));
+                                Qd = mul2(s2, fma2(a3, y[2][m], Qd));
+                                if constexpr (MODE == 1) {
+                                    outv[m] = Qd;
+                                } else {
+                                    float2 B = fma2(ee, y[0][m], make_float2(-y[1][m].x, -y[1][m].y));
+                                    B = fma2(mul2(f2(2.f), fv), y[2][m], B);
+                                    outv[m] = mul2(mul2(u, u), B);
+                                    part = fma2(so[m], B, part);
+                                    outq[m] = Qd;
+                                }
+                            }
+                        }
+                        if constexpr (OUT_X) {
+                            // caller layout: rows of W values, 8-byte aligned when W is even (and the
+                            // caller's base is), then one 8-byte store per pair
+                            const Geom& g = P.g;
+                            const int h = r.h0 + row, wb = r.w0 + seg * 8;
+                            float* o = reinterpret_cast<float*>(P.out) + ((int64_t)to * g.H + h) * g.W + wb;
+                            if (h < g.H) {
+                                if (wb + 8 <= g.W && (reinterpret_cast<uintptr_t>(o) & 7) == 0) {
+#pragma unroll
+                                    for (int m = 0; m < 4; ++m) reinterpret_cast<float2*>(o)[m] = outv[m];
+                                } else {
+#pragma unroll
+                                    for (int m = 0; m < 4; ++m) {
+                                        if (wb + 2 * m < g.W) o[2 * m] = outv[m].x;
+                                        if (wb + 2 * m + 1 < g.W) o[2 * m + 1] = outv[m].y;
+                                    }
+                                }
+                            }
+                        } else {
+                            st_cols(reinterpret_cast<TVO*>(smem + C::O_O + b * C::OT) + tile_off, outv);
+                        }
+                        if constexpr (E::OUT2) st_cols(reinterpret_cast<float*>(smem + C::O_O2 + b * C::T32) + tile_off, outq);
+                    }
+                    fence_async();       // the tiles written here are read by TMA stores
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&done[b]);
+                    ++e;
                 }
-                fence_async();       // the tiles written here are read by TMA stores
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&done[b]);
-                ++e;
+            };
+            if constexpr (kFoldInside) {
+                frames(r.t1);
+            } else {
+#pragma unroll 1
+                while (ok && to < r.t1) {
+                    fold();
+                    frames(min(r.t1, to + kFold));
+                }
             }
         }
         red[i] += (double)part.x + (double)part.y;

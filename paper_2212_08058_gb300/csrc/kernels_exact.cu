@@ -6,12 +6,11 @@
 // the next x~ = A S / a.  The norm s = 1/||x~|| is summed by the pass that forms w and applied by the
 // filtering (the operator is linear), so no pass waits for it.
 //
-// c = 0 is the series in f itself.  The middle of f's range halves max |g|, and the terms needed
-// follow x = 2 a max(g)^2: 9 instead of 16 for f in [0, 1] at a = 1, three filterings a step instead of
-// six.  These passes move 12 bytes per voxel, four columns per thread (rows start 128-byte aligned);
-// forming each group's input from x~ with the power and the exponential took 12 bytes and, with the
-// norm's FP64 in every thread, 28.6 us for 3.3M voxels.  Five steps at 32x240x427, (2,7,7), the call:
-// 1449 us with the series in f, 659 us now.
+// c = 0 is the series in f itself, which g reads then.  The middle of f's range halves max |g|, and the terms
+// needed follow x = 2 a max(g)^2: 9 instead of 16 for f in [0, 1] at a = 1, three filterings a step instead
+// of six, but its alternating terms cancel digits of small outputs, so it is taken up to
+// a (range of f)^2 = 1 (kCentredRange, api.cu).  These passes move 12 bytes per voxel, four columns per
+// thread (rows start 128-byte aligned).  Five steps at 32x240x427, (2,7,7), the call: 621 us centred.
 #include "launch.h"
 #include "order_key.cuh"
 #include "tma.cuh"
