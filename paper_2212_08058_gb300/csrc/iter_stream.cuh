@@ -33,7 +33,7 @@
 // address space, so that every access is a generic one: the alignment is an offset (152 us per step; 184
 // through an integer).
 // Measured per step, small-volume kernel / this one: (2,7,7) 64x480x854 168 / 138 us (the algorithmic
-// multiply-adds alone 68 us), 120x1080x1920 1163 here; (1,3,3) 64x480x854 111 / 95.
+// multiply-adds alone 68 us), 120x1080x1920 1170 here; (1,3,3) 64x480x854 111 / 94.
 #pragma once
 
 #include "order_key.cuh"

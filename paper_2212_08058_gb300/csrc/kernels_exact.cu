@@ -10,7 +10,8 @@
 // needed follow x = 2 a max(g)^2: 9 instead of 16 for f in [0, 1] at a = 1, three filterings a step instead
 // of six, but its alternating terms cancel digits of small outputs, so it is taken up to
 // a (range of f)^2 = 1 (kCentredRange, api.cu).  These passes move 12 bytes per voxel, four columns per
-// thread (rows start 128-byte aligned).  Five steps at 32x240x427, (2,7,7), the call: 621 us centred.
+// thread (rows start 128-byte aligned).  Five steps at 32x240x427, (2,7,7), f in [0, 1], the call: 597 us
+// centred, 1097 with the series in f.
 #include "launch.h"
 #include "order_key.cuh"
 #include "tma.cuh"
