@@ -28,10 +28,17 @@ class _Full:
     def __enter__(self):
         torch.cuda.synchronize()
         torch.cuda.empty_cache()
-        self.block = torch.empty(torch.cuda.mem_get_info()[0] - self.leave, device="cuda", dtype=torch.uint8)
+        self.blocks = []
+        step = torch.cuda.mem_get_info()[0] - self.leave
+        while step >= 20 * MB:       # one block, or smaller ones where the free memory is in pieces
+            try:
+                self.blocks.append(torch.empty(step, device="cuda", dtype=torch.uint8))
+            except torch.OutOfMemoryError:
+                step //= 2
+            step = min(step, torch.cuda.mem_get_info()[0] - self.leave)
 
     def __exit__(self, *exc):
-        del self.block
+        del self.blocks
         torch.cuda.empty_cache()
 
 
