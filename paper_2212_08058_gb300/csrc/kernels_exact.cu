@@ -42,8 +42,19 @@ RowLaunch quad_launch(const Geom& g, int per_sm) {
     return {(int)(rows < cap ? rows : cap), w4 >= 128 ? 128 : (w4 + 31) / 32 * 32};
 }
 
-__device__ __forceinline__ void add_sum(float part, double* acc) {
-    const double b = block_sum((double)part);
+// A thread's sum of squares, each addition's rounding carried into the next (Kahan).  A plain float32 sum
+// takes 850 terms of a 120x1080x1920 volume and put the norm of equal voxels 8e-6 off.
+struct SquareSum {
+    float s = 0.f, c = 0.f;
+    __device__ __forceinline__ void add(float v) {
+        const float y = __fmaf_rn(v, v, -c), t = __fadd_rn(s, y);
+        c = __fsub_rn(__fsub_rn(t, s), y);
+        s = t;
+    }
+};
+
+__device__ __forceinline__ void add_sum(const SquareSum& part, double* acc) {
+    const double b = block_sum((double)part.s - (double)part.c);
     if (threadIdx.x == 0 && acc) atomicAdd(acc, b);
 }
 
@@ -78,21 +89,21 @@ __global__ void exact_setup_kernel(const float* f, float center, float alpha, fl
 }
 
 __global__ void exact_in_kernel(const float* x_user, const float* A, Geom g, float* w, double* acc) {
-    float part = 0.f;
+    SquareSum part;
     for_each_voxel(g, [&](int64_t i, int64_t j) {
         const float v = x_user ? x_user[i] : 1.f;
         w[j] = A[j] * v;
-        part += v * v;
+        part.add(v);
     });
     add_sum(part, acc);
 }
 
 __global__ void exact_mid_kernel(const float* S, const float* A, float inv_alpha, Geom g, float* w, double* acc) {
     wait_previous_grid();
-    float part = 0.f;
+    SquareSum part;
     auto one = [&](float s, float a) {
         const float x = a * s * inv_alpha;
-        part += x * x;
+        part.add(x);
         return a * x;
     };
     for_each_quad(
@@ -118,11 +129,11 @@ __global__ void exact_next_kernel(const float* gf, Geom g, float* v) {
 }
 
 __global__ void exact_out_kernel(const float* S, const float* A, float inv_alpha, Geom g, float* x_user, double* acc) {
-    float part = 0.f;
+    SquareSum part;
     for_each_voxel(g, [&](int64_t i, int64_t j) {
         const float x = A[j] * S[j] * inv_alpha;
         x_user[i] = x;
-        part += x * x;
+        part.add(x);
     });
     add_sum(part, acc);
 }

@@ -181,3 +181,19 @@ def test_no_exact_steps_is_the_normalised_start(sf, T, H, W):
         with pytest.raises(sf.SFSegError) as e:
             h.power_iterate_exact((1, 3, 3), iters=0, x=torch.zeros_like(x), init="user", return_norms=True)
         assert e.value.status == "ZERO_NORM"
+
+
+def test_exact_norm_of_many_equal_voxels(sf):
+    """The norms of the exact operator on 120x1080x1920 equal voxels.  A thread's sum carries its own
+    roundings, 2 of 2^-24 in all, and the outputs' own (17 taps, two equal sides of an edge, 8 for u, the
+    exponential and the combination) are common to the reference: (2 + 8) / 2 * 2^-24 = 3e-7, and as much
+    for the float32 reciprocal norm of each step."""
+    T, H, W, r = 120, 1080, 1920, (1, 3, 3)
+    with sf.PowerIteration(1, T, H, W) as h:
+        h.set_features(torch.full((1, T, H, W), 0.6, device="cuda"))
+        _, nu = h.power_iterate_exact(r, iters=2, return_norms=True)
+        y = h.apply_exact(torch.full((T, H, W), (T * H * W) ** -0.5, device="cuda"), r)
+        n1 = float(y.double().norm())
+        y.mul_(1.0 / n1)
+        n2 = float(h.apply_exact(y, r).double().norm())
+    assert abs(nu[0] / n1 - 1.0) <= 6e-7 and abs(nu[1] / n2 - 1.0) <= 6e-7
