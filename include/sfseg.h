@@ -178,7 +178,9 @@ int sfseg_rayleigh(sfseg_handle* h, const sfseg_neighborhood* nb, const float* x
  * on this handle (which must have used record_every > 0, C > 1, and features != NULL or set),
  * write dL/dw (host, C floats) and dL/db (host, 1 float).  The adjoint runs backwards through
  * the K normalised steps, recomputing iterates between checkpoints.  Synchronises.
- * Errors: STATE (no recorded forward), UNSUPPORTED (C == 1, or bf16 iterations recorded). */
+ * Workspace, allocated on first use: record_every + 4 volumes, and for rt <= 2 another
+ * record_every + 3 (a radius without a kernel of its own does without these if they do not fit).
+ * Errors: STATE (no recorded forward), UNSUPPORTED (C == 1, or bf16 iterations recorded), OOM. */
 int sfseg_backward(sfseg_handle* h, const sfseg_neighborhood* nb, const float* grad_x,
                    float* grad_weights, float* grad_bias, void* stream);
 
